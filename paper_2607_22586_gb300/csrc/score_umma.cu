@@ -68,69 +68,90 @@ struct Sched {
   WorkLists wl;
 };
 
-// A worker's walk over its list, one split row at a time. The plain team
-// schedule is resolved once: a = the worker's first split row, c = its
-// block. A list is followed segment by segment: c = current segment, a =
-// split rows of the worker before it. LISTS (a template argument of both
-// kernels) selects the list form at compile time, so the plain-team kernels
-// carry no list walk.
+// A worker's walk over its units, one split row at a time: the current unit
+// (layer, request, KV head, key split, stationary block) and what its keys
+// need. A team's rows and a list's segments are runs of consecutive split
+// rows, so only the first unit of a run is decoded from its index (five
+// integer divisions); the next ones follow by counting up. Decoding every
+// unit cost an epilogue warp about as many instructions as the exponentials
+// of one of the unit's tiles. LISTS (a template argument of both kernels)
+// selects the list form at compile time.
 struct Walk {
-  int n;      // split rows of the worker
-  int a, c;
+  int seg, left;                 // current run, its rows after this one
+  int l, b, h, split, tile;      // the unit
+  int nsplit, t_len, tok_off;    // of request b
+  bool fresh;                    // first unit of a (layer, request, KV head, block)
+  int t0, t1;                    // its keys
 };
 
-template <bool LISTS>
-__device__ __forceinline__ Walk walk_begin(const Sched& S, int w, int nw) {
+__device__ __forceinline__ Walk walk_begin() {
   Walk k;
-  if (LISTS) {
-    k.n = 0;
-    for (int i = 0; i < S.wl.nseg[w]; ++i) k.n += S.wl.seg[w][i].e - (S.wl.seg[w][i].bt >> 8);
-    k.a = 0;
-    k.c = 0;
-  } else {
-    const int nteams = nw / S.ntiles, team = w / S.ntiles;
-    const int rows = S.units / S.ntiles;
-    k.a = (int)((long long)team * rows / nteams);
-    k.n = (int)((long long)(team + 1) * rows / nteams) - k.a;
-    k.c = w % S.ntiles;
-  }
+  k.seg = -1;
+  k.left = 0;
   return k;
 }
 
-// Unit index of the worker's i-th split row; i grows by one per call.
-template <bool LISTS>
-__device__ __forceinline__ int walk_unit(const Sched& S, int w, Walk& k, int i) {
-  if (!LISTS) return (k.a + i) * S.ntiles + k.c;
-  for (;;) {
-    const PackedSeg p = S.wl.seg[w][k.c];
-    const int b = p.bt >> 8, len = p.e - b;
-    if (i - k.a < len) return (b + i - k.a) * S.ntiles + (p.bt & 255);
-    k.a += len;
-    ++k.c;
-  }
+__device__ __forceinline__ void walk_request(const Problem& P, Walk& k) {
+  k.nsplit = P.req[k.b].nsplit;
+  k.t_len = P.req[k.b].t_len;
+  k.tok_off = P.req[k.b].tok_off;
 }
 
-struct Unit {
-  int l, b, h, tile, split, t0, t1;
-};
-
-__device__ __forceinline__ Unit decode(const Problem& P, const Sched& S, int u) {
-  Unit x;
-  const int per_layer = S.uoff[P.B];
-  x.l = u / per_layer;
-  int r = u - x.l * per_layer;
+// First unit of a run: split row `row` of stationary block `tile`.
+__device__ __forceinline__ void walk_seek(const Problem& P, const Sched& S, Walk& k, int row,
+                                          int tile) {
+  const int per_layer = S.uoff[P.B] / S.ntiles;
+  k.tile = tile;
+  k.l = row / per_layer;
+  int r = row - k.l * per_layer;
   int b = 0;
-  while (b + 1 < P.B && S.uoff[b + 1] <= r) ++b;
-  x.b = b;
-  r -= S.uoff[b];
-  const int ns = P.req[b].nsplit;
-  x.tile = r % S.ntiles;
-  r /= S.ntiles;
-  x.split = r % ns;
-  x.h = r / ns;
-  x.t0 = x.split * P.split_len;
-  x.t1 = min(P.req[b].t_len, x.t0 + P.split_len);
-  return x;
+  while (b + 1 < P.B && S.uoff[b + 1] / S.ntiles <= r) ++b;
+  k.b = b;
+  r -= S.uoff[b] / S.ntiles;
+  walk_request(P, k);
+  k.h = r / k.nsplit;
+  k.split = r - k.h * k.nsplit;
+  k.fresh = true;
+}
+
+// The worker's next unit; false when it has none left.
+template <bool LISTS>
+__device__ __forceinline__ bool walk_next(const Problem& P, const Sched& S, int w, int nw, Walk& k) {
+  if (k.left > 0) {
+    --k.left;
+    k.fresh = false;
+    if (++k.split == k.nsplit) {
+      k.split = 0;
+      k.fresh = true;
+      if (++k.h == P.Hkv) {
+        k.h = 0;
+        if (++k.b == P.B) { k.b = 0; ++k.l; }
+        walk_request(P, k);
+      }
+    }
+  } else if (LISTS) {
+    for (;;) {
+      if (++k.seg >= S.wl.nseg[w]) return false;
+      const PackedSeg p = S.wl.seg[w][k.seg];
+      const int b = p.bt >> 8, n = p.e - b;
+      if (n <= 0) continue;
+      walk_seek(P, S, k, b, p.bt & 255);
+      k.left = n - 1;
+      break;
+    }
+  } else {
+    if (++k.seg > 0) return false;
+    const int nteams = nw / S.ntiles, team = w / S.ntiles;
+    const int rows = S.units / S.ntiles;
+    const int a = (int)((long long)team * rows / nteams);
+    const int n = (int)((long long)(team + 1) * rows / nteams) - a;
+    if (n <= 0) return false;
+    walk_seek(P, S, k, a, w % S.ntiles);
+    k.left = n - 1;
+  }
+  k.t0 = k.split * P.split_len;
+  k.t1 = min(k.t_len, k.t0 + P.split_len);
+  return true;
 }
 
 // Rows of stationary block t of the mass pass. Blocks hold whole groups;
@@ -160,10 +181,6 @@ __host__ __device__ inline Block mass_block(const Problem& P, const Sched& S, in
   return k;
 }
 
-__device__ __forceinline__ long long block_key(const Problem& P, const Sched& S, const Unit& x) {
-  return ((long long)(x.l * P.B + x.b) * P.Hkv + x.h) * S.ntiles + x.tile;
-}
-
 template <int D>
 struct Smem {
   static constexpr int CH = D / 64;                         // 128-byte K chunks
@@ -185,7 +202,7 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
 // The max is only raised when the chunk's sum relative to it would exceed
 // 2^100 (or while it is still -inf), so the common path is FFMA + EX2 + FADD; z
 // stays below 2^127 over the 32 chunks of a key split.
-__device__ __noinline__ void mask_tail(float (&v)[32], int c0, int nvalid) {
+__device__ __forceinline__ void mask_tail(float (&v)[32], int c0, int nvalid) {
 #pragma unroll
   for (int j = 0; j < 32; ++j)
     if (c0 + j >= nvalid) v[j] = -INFINITY;
@@ -270,12 +287,27 @@ __device__ __forceinline__ void mass_chunk(const float (&v)[16], const uint64_t 
 }
 
 // Sum over the ncols (multiple of 8) accumulator columns of one group:
-// sum_j exp2(acc_j * alpha - c_j), four partial sums added in a fixed order.
-// nc points at the warp's shared-memory copy of the block's negated normalisers.
-__device__ __forceinline__ float group_sum(uint32_t tcol, const float* nc, int ncols, float alpha) {
+// sum_j exp2(acc_j * alpha - c_j), column j feeding partial sum j mod 4 in
+// ascending order (the odd 16 columns first, so that the last load is a wide
+// one), the four partial sums added in a fixed order. nc points at the warp's
+// shared-memory copy of the block's negated normalisers; loaded() runs once,
+// when the last columns are in registers and before their exponentials.
+template <class Loaded>
+__device__ __forceinline__ float group_sum(uint32_t tcol, const float* nc, int ncols, float alpha,
+                                           const Loaded& loaded) {
   const uint64_t al2 = pk2(alpha, alpha);
   uint64_t a01 = 0, a23 = 0;       // (+0, +0)
   int cc = 0;
+  if (ncols & 16) {
+    float v[16];
+    uint64_t ncv[8];
+    tmem_ld16(tcol, v);
+    load_nc16(nc, ncv);
+    tmem_wait_ld();
+    if (ncols == 16) loaded();
+    mass_chunk(v, ncv, al2, a01, a23);
+    cc = 16;
+  }
 #pragma unroll 1
   for (; cc + 32 <= ncols; cc += 32) {
     float v[32];
@@ -283,18 +315,10 @@ __device__ __forceinline__ float group_sum(uint32_t tcol, const float* nc, int n
     tmem_ld32(tcol + cc, v);
     load_nc16(nc + cc, ncv);
     tmem_wait_ld();
+    if (cc + 32 == ncols) loaded();
     mass_chunk(*reinterpret_cast<float(*)[16]>(v), ncv, al2, a01, a23);
     load_nc16(nc + cc + 16, ncv);
     mass_chunk(*reinterpret_cast<float(*)[16]>(v + 16), ncv, al2, a01, a23);
-  }
-  if (cc + 16 <= ncols) {
-    float v[16];
-    uint64_t ncv[8];
-    tmem_ld16(tcol + cc, v);
-    load_nc16(nc + cc, ncv);
-    tmem_wait_ld();
-    mass_chunk(v, ncv, al2, a01, a23);
-    cc += 16;
   }
   if (cc < ncols) {   // an 8-column tail (the anchor rows, r <= 8)
     float v[8];
@@ -302,6 +326,7 @@ __device__ __forceinline__ float group_sum(uint32_t tcol, const float* nc, int n
     const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(nc + cc);
     const ulonglong2 n0 = c2[0], n1 = c2[1];
     tmem_wait_ld();
+    loaded();
     float y0, y1, y2, y3;
     upk2(ffma2(pk2(v[0], v[1]), al2, n0.x), y0, y1);
     upk2(ffma2(pk2(v[2], v[3]), al2, n0.y), y2, y3);
@@ -343,7 +368,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // a CTA reloads its stationary block only when the (layer, request, head)
   // or the block changes. The three roles walk the same list.
   const int wk = blockIdx.x;
-  Walk walk = walk_begin<LISTS>(S, wk, gridDim.x);
+  const int nwk = gridDim.x;
+  Walk x = walk_begin();
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -355,7 +381,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     mbar_init(&sempty, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&tfull[i], 1);
-      mbar_init(&tempty[i], NEPI / 2);   // drained by a pair of warpgroups
+      mbar_init(&tempty[i], NEPI / 2 / 32);   // the warps of a pair of warpgroups
     }
     mbar_init(&drain, 1);
     mbar_init(&never, 1);                // nothing arrives here (test_stuck_wait)
@@ -378,13 +404,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       int stage = 0;
       uint32_t phase = 0, sphase = 0;
       ArmedStages armed_k, armed_s;
-      long long prev = -1;
       bool ok = true;
-      for (int i = 0; i < walk.n && ok; ++i) {
-        const int u = walk_unit<LISTS>(S, wk, walk, i);
-        const Unit x = decode(P, S, u);
-        const long long key = block_key(P, S, x);
-        if (key != prev) {
+      while (ok && walk_next<LISTS>(P, S, wk, nwk, x)) {
+        if (x.fresh) {
           if (!mbar_wait(&sempty, sphase ^ 1u, abort_)) { ok = false; break; }
           const Block k = mass_block(P, S, x.tile);
           const int row0 = k.row0, rows = k.rows;
@@ -395,9 +417,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             for (int r = 0; r < rows; r += 16)
               tma_load_3d(stat + c * SROWS * 128 + r * 128, &pmap, &sfull, c * 64, row0 + r, zc);
           sphase ^= 1u;
-          prev = key;
         }
-        const int kbase = P.req[x.b].tok_off;
+        const int kbase = x.tok_off;
         for (int kt = x.t0; kt < x.t1; kt += BK) {
           if (!mbar_wait(&empty[stage], phase ^ 1u, abort_)) { ok = false; break; }
           mbar_expect_tx(&full[stage], (uint32_t)SM::STAGE_BYTES);
@@ -416,20 +437,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     if (lane == 0) {
       int stage = 0;
       uint32_t phase = 0, bphase = 0, sphase = 0;   // bphase: one phase bit per accumulator
-      long long prev = -1;
       uint32_t idesc = 0;
       bool ok = true, issued = false;
-      for (int i = 0; i < walk.n && ok; ++i) {
-        const int u = walk_unit<LISTS>(S, wk, walk, i);
-        const Unit x = decode(P, S, u);
-        const long long key = block_key(P, S, x);
-        if (key != prev) {
-          if (prev != -1) mma_commit(&sempty);   // old block free once its MMAs finish
+      while (ok && walk_next<LISTS>(P, S, wk, nwk, x)) {
+        if (x.fresh) {
+          if (issued) mma_commit(&sempty);   // old block free once its MMAs finish
           if (!mbar_wait(&sfull, sphase, abort_)) { ok = false; break; }
           sphase ^= 1u;
           fence_after();
           idesc = idesc_bf16_f32(128, mass_block(P, S, x.tile).rows);
-          prev = key;
         }
         // accumulator = parity of the tile's index within its split, so a
         // split's tiles reach the same epilogue warpgroups whatever ran before
@@ -474,53 +490,60 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int lrow = q * 32 + lane;       // accumulator lane: a key of the tile
     const float alpha = P.alpha;
     uint32_t bphase = 0;                  // one phase bit per accumulator
-    long long prev_blk = -1;
     bool ok = true;
     // test only: the first epilogue warp of CTA 0 waits on a barrier that
     // nothing arrives on, gives up after a few polls and aborts the CTA
     if (P.test_stuck_wait && blockIdx.x == 0 && ew == 0)
       ok = mbar_wait(&never, 0, abort_, kTestSpinLimit);
-    for (int i = 0; i < walk.n && ok; ++i) {
-      const int u = walk_unit<LISTS>(S, wk, walk, i);
-      const Unit x = decode(P, S, u);
-      const ReqInfo R = P.req[x.b];
-      const long long key = block_key(P, S, x);
-      const Block blk = mass_block(P, S, x.tile);
-      const float* cv = cs_all + ew * SROWS;   // this warp's copy of the block's negated normalisers
-      if (key != prev_blk) {
+    const float* cv = cs_all + ew * SROWS;   // this warp's copy of the block's negated normalisers
+    Block blk{};
+    int gb = 0, ge = 0;                      // this warpgroup's groups of the block
+    bool my_anchor = false;
+    float* gdst = nullptr;                   // mass row of group gb, this thread's key lane
+    while (ok && walk_next<LISTS>(P, S, wk, nwk, x)) {
+      if (x.fresh) {
+        blk = mass_block(P, S, x.tile);
+        const int ng0 = (blk.ng + 1) / 2;
+        gb = sub == 0 ? 0 : ng0;
+        ge = sub == 0 ? ng0 : blk.ng;
+        my_anchor = blk.anchor && (blk.ng == 0 ? sub == 0 : sub == 1);
         const float* src = bf.cvals + (((size_t)x.l * P.B + x.b) * P.Hkv + x.h) * P.Prows_pad + blk.row0;
         __syncwarp();
         for (int i = lane; i < blk.rows; i += 32) cs_all[ew * SROWS + i] = -src[i];
         __syncwarp();
-        prev_blk = key;
+        gdst = bf.gmass + (((size_t)x.l * P.Hkv + x.h) * P.G + blk.g0 + gb) * P.total_T +
+               x.tok_off + lrow;
       }
-      for (int kt = x.t0, j = 0; kt < x.t1; kt += BK, ++j) {
-        const int buf = j & 1;
-        if (buf != par) continue;
+      for (int kt = x.t0 + par * BK, buf = par; kt < x.t1; kt += 2 * BK) {
         const uint32_t ph = (bphase >> buf) & 1u;
         bphase ^= 1u << buf;
         if (!mbar_wait(&tfull[buf], ph, abort_)) { ok = false; break; }
         fence_after();
         const uint32_t tacc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * ACC_STRIDE);
-        const int t = kt + lrow;
-        const bool valid = t < x.t1;
-        const size_t col = (size_t)R.tok_off + t;
-        const int ng0 = (blk.ng + 1) / 2;
-        const int gb = sub == 0 ? 0 : ng0, ge = sub == 0 ? ng0 : blk.ng;
-        for (int gi = gb; gi < ge; ++gi) {
-          const float sm = group_sum(tacc + (uint32_t)(gi * P.RG), cv + gi * P.RG, P.RG, alpha);
-          if (valid)
-            bf.gmass[(((size_t)x.l * P.Hkv + x.h) * P.G + blk.g0 + gi) * P.total_T + col] = sm;
+        const bool valid = kt + lrow < x.t1;
+        // released once this warp's last columns are in registers
+        auto release = [&] {
+          fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&tempty[buf]);
+        };
+        float* out = gdst + kt;
+        for (int gi = gb; gi < ge; ++gi, out += P.total_T) {
+          const bool last = gi + 1 == ge && !my_anchor;
+          const float sm = group_sum(tacc + (uint32_t)(gi * P.RG), cv + gi * P.RG, P.RG, alpha,
+                                     [&] { if (last) release(); });
+          if (valid) *out = sm;
         }
-        const bool my_anchor = blk.anchor && (blk.ng == 0 ? sub == 0 : sub == 1);
         if (my_anchor) {
           const int a0 = blk.ng * P.RG;
+          const size_t col = (size_t)x.tok_off + kt + lrow;
           if (P.anchor_split) {
             // no normalisers yet: the scaled logits go to alog, row by row
             // (coalesced along keys), for anchor_part_kernel / anchor_final_kernel
             float v[kMaxSplitAnchor];
             tmem_ld8(tacc + (uint32_t)a0, v);
             tmem_wait_ld();
+            release();
             if (valid) {
               float* dst = bf.alog + ((size_t)x.l * P.Hkv + x.h) * P.r * P.total_T + col;
 #pragma unroll
@@ -530,13 +553,13 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           } else {
             // the r anchor rows, in 8-column steps (the padding rows up to 16
             // would add exp2(-inf) = 0)
-            const float sm = group_sum(tacc + (uint32_t)a0, cv + a0, (P.r + 7) & ~7, alpha);
+            const float sm = group_sum(tacc + (uint32_t)a0, cv + a0, (P.r + 7) & ~7, alpha, release);
             if (valid)
               bf.anchor[((size_t)x.l * P.Hkv + x.h) * P.total_T + col] = sm / (float)P.r;
           }
+        } else if (gb == ge) {
+          release();   // no columns of this block
         }
-        fence_before();
-        mbar_arrive(&tempty[buf]);
       }
     }
   }
@@ -597,7 +620,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
   const uint32_t rank = cluster_rank();
   // work lists as in the one-SM kernel, one per pair
   const int wk = blockIdx.x >> 1;
-  Walk walk = walk_begin<LISTS>(S, wk, gridDim.x >> 1);
+  const int nwk = gridDim.x >> 1;
+  Walk x = walk_begin();
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -632,12 +656,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
       int stage = 0;
       uint32_t phase = 0, sphase = 0;
       ArmedStages armed_k, armed_s;   // the leader's barriers count both CTAs' loads
-      long long prev = -1;
       bool ok = true;
-      for (int i = 0; i < walk.n && ok; ++i) {
-        const Unit x = decode(P, S, walk_unit<LISTS>(S, wk, walk, i));
-        const long long key = block_key(P, S, x);
-        if (key != prev) {
+      while (ok && walk_next<LISTS>(P, S, wk, nwk, x)) {
+        if (x.fresh) {
           if (!mbar_wait(&sempty, sphase ^ 1u, abort_)) { ok = false; break; }
           if (rank == 0) {
             mbar_expect_tx(&sfull, (uint32_t)(2 * PROWS * D * 2));
@@ -650,9 +671,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             for (int r = 0; r < PROWS; r += 16)
               tma_load_3d_pair(stat + c * PROWS * 128 + r * 128, &pmap, bar, c * 64, row0 + r, zc);
           sphase ^= 1u;
-          prev = key;
         }
-        const int kbase = P.req[x.b].tok_off + (int)rank * (PBK / 2);
+        const int kbase = x.tok_off + (int)rank * (PBK / 2);
         for (int kt = x.t0; kt < x.t1; kt += PBK) {
           if (!mbar_wait(&empty[stage], phase ^ 1u, abort_)) { ok = false; break; }
           if (rank == 0) {
@@ -675,18 +695,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     if (lane == 0 && rank == 0) {
       int stage = 0;
       uint32_t phase = 0, bphase = 0, sphase = 0;
-      long long prev = -1;
       const uint32_t idesc = idesc_bf16_f32(2 * PROWS, PBK);
       bool ok = true, issued = false;
-      for (int i = 0; i < walk.n && ok; ++i) {
-        const Unit x = decode(P, S, walk_unit<LISTS>(S, wk, walk, i));
-        const long long key = block_key(P, S, x);
-        if (key != prev) {
-          if (prev != -1) mma_commit_pair(&sempty, 0x3);   // old block free once its MMAs finish
+      while (ok && walk_next<LISTS>(P, S, wk, nwk, x)) {
+        if (x.fresh) {
+          if (issued) mma_commit_pair(&sempty, 0x3);   // old block free once its MMAs finish
           if (!mbar_wait(&sfull, sphase, abort_)) { ok = false; break; }
           sphase ^= 1u;
           fence_after();
-          prev = key;
         }
         for (int kt = x.t0, j = 0; kt < x.t1; kt += PBK, ++j) {
           const int buf = j & 1;
@@ -727,13 +743,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     const uint32_t tempty_lead[2] = {mapa(smem_u32(&tempty[0]), 0), mapa(smem_u32(&tempty[1]), 0)};
     uint32_t bphase = 0;
     bool ok = true;
-    for (int i = 0; i < walk.n && ok; ++i) {
-      const Unit x = decode(P, S, walk_unit<LISTS>(S, wk, walk, i));
-      const ReqInfo R = P.req[x.b];
+    float2* dst = nullptr;
+    while (ok && walk_next<LISTS>(P, S, wk, nwk, x)) {
+      const size_t dst_step = (size_t)kUmmaPartSlots * P.Prows_pad;
+      if (x.fresh)
+        dst = bf.part + (((size_t)x.l * P.Hkv + x.h) * P.total_splits + P.req[x.b].split_off + x.split) * dst_step +
+              (size_t)wg * P.Prows_pad + x.tile * SROWS + (int)rank * PROWS + lrow;
+      else
+        dst += dst_step;
       // (reference max, sum of exp2(x - max)) of this thread's row over its
       // quarter of every tile of the split, restarted per split
       float m_run = -INFINITY, z_run = 0.f;
-      bool first = true;
       for (int kt = x.t0, j = 0; kt < x.t1; kt += PBK, ++j) {
         const int buf = j & 1;
         const uint32_t ph = (bphase >> buf) & 1u;
@@ -743,42 +763,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         const uint32_t tcol =
             tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * PBK + c_lo);
         const int nvalid = min(PBK, x.t1 - kt) - c_lo;
-        if (nvalid >= PBK / 4) {         // every tile but the last of a short split
+        // the accumulator is released as soon as its last columns are in
+        // registers, before their exponentials, so the MMAs of the tile after
+        // next start half a drain earlier
 #pragma unroll 1
-          for (int c0 = 0; c0 < PBK / 4; c0 += 32) {
-            float v[32];
-            tmem_ld32(tcol + c0, v);
-            tmem_wait_ld();
-            if (first) {
-              softmax_first(v, alpha, m_run, z_run);
-              first = false;
-            } else {
-              softmax_chunk(v, alpha, m_run, z_run);
-            }
+        for (int c0 = 0; c0 < PBK / 4; c0 += 32) {
+          float v[32];
+          tmem_ld32(tcol + c0, v);
+          tmem_wait_ld();
+          if (c0 == PBK / 4 - 32) {
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster_relaxed(tempty_lead[buf]);
           }
-        } else {
-#pragma unroll 1
-          for (int c0 = 0; c0 < PBK / 4; c0 += 32) {
-            float v[32];
-            tmem_ld32(tcol + c0, v);
-            tmem_wait_ld();
-            mask_tail(v, c0, nvalid);
-            if (first) {
-              softmax_first(v, alpha, m_run, z_run);
-              first = false;
-            } else {
-              softmax_chunk(v, alpha, m_run, z_run);
-            }
-          }
+          if (nvalid < PBK / 4) mask_tail(v, c0, nvalid);   // the last tile of a short split
+          if (j == 0 && c0 == 0)
+            softmax_first(v, alpha, m_run, z_run);
+          else
+            softmax_chunk(v, alpha, m_run, z_run);
         }
-        fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster_relaxed(tempty_lead[buf]);
       }
       if (!ok) break;
-      const int prow = x.tile * SROWS + (int)rank * PROWS + lrow;
-      bf.part[((((size_t)x.l * P.Hkv + x.h) * P.total_splits + R.split_off + x.split) * kUmmaPartSlots +
-               wg) * P.Prows_pad + prow] = make_float2(m_run, z_run);
+      *dst = make_float2(m_run, z_run);
     }
   }
 
