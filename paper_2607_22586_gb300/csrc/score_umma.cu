@@ -228,14 +228,23 @@ __device__ __forceinline__ float exp2_sum32(const float (&v)[32], uint64_t al2, 
   return (s0 + s1) + (s2 + s3);
 }
 
+// Largest of 32 logits. Scaling it equals the largest scaled logit: alpha > 0
+// and rounding to nearest keeps the order.
+__device__ __forceinline__ float max32(const float (&v)[32]) {
+  float c0 = v[0], c1 = v[1];
+#pragma unroll
+  for (int j = 2; j < 32; j += 2) {
+    c0 = fmaxf(c0, v[j]);
+    c1 = fmaxf(c1, v[j + 1]);
+  }
+  return fmaxf(c0, c1);
+}
+
 __device__ __forceinline__ void softmax_chunk(float (&v)[32], float alpha, float& m, float& z) {
   const uint64_t al2 = pk2(alpha, alpha);
   float zc = exp2_sum32(v, al2, m);
   if (!(zc <= 1.2676506e30f)) {  // first chunk, sum above 2^100 or NaN: raise the max
-    float cm = -INFINITY;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) cm = fmaxf(cm, v[j] * alpha);
-    const float mn = fmaxf(m, cm);
+    const float mn = fmaxf(m, max32(v) * alpha);
     if (mn == -INFINITY) {
       zc = 0.f;
     } else {
@@ -250,26 +259,16 @@ __device__ __forceinline__ void softmax_chunk(float (&v)[32], float alpha, float
 // First chunk of a split: the reference is the chunk's own max (ALU only, so
 // the exponentials are evaluated once); z starts from this chunk's sum.
 __device__ __forceinline__ void softmax_first(const float (&v)[32], float alpha, float& m, float& z) {
-  float c0 = -INFINITY, c1 = -INFINITY;
-#pragma unroll
-  for (int j = 0; j < 32; j += 2) {
-    c0 = fmaxf(c0, v[j] * alpha);
-    c1 = fmaxf(c1, v[j + 1] * alpha);
-  }
-  m = fmaxf(c0, c1);
+  m = max32(v) * alpha;
   if (m == -INFINITY) return;      // every column masked: nothing to add
   z = exp2_sum32(v, pk2(alpha, alpha), m);
 }
 
 // 16 consecutive negated row normalisers (-c) from the warp's shared-memory
 // copy, as 8 packed pairs.
-__device__ __forceinline__ void load_nc16(const float* nc, uint64_t (&ncv)[8]) {
-  const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(nc);
+__device__ __forceinline__ void load_nc16(uint32_t nc, uint64_t (&ncv)[8]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const ulonglong2 t = c2[i];
-    ncv[2 * i] = t.x; ncv[2 * i + 1] = t.y;
-  }
+  for (int i = 0; i < 4; ++i) lds_2x64(nc + 16 * i, ncv[2 * i], ncv[2 * i + 1]);
 }
 
 // a01 += (e_j, e_j+1), a23 += (e_j+2, e_j+3) over 16 columns, e_j =
@@ -293,7 +292,7 @@ __device__ __forceinline__ void mass_chunk(const float (&v)[16], const uint64_t 
 // shared-memory copy of the block's negated normalisers; loaded() runs once,
 // when the last columns are in registers and before their exponentials.
 template <class Loaded>
-__device__ __forceinline__ float group_sum(uint32_t tcol, const float* nc, int ncols, float alpha,
+__device__ __forceinline__ float group_sum(uint32_t tcol, uint32_t nc, int ncols, float alpha,
                                            const Loaded& loaded) {
   const uint64_t al2 = pk2(alpha, alpha);
   uint64_t a01 = 0, a23 = 0;       // (+0, +0)
@@ -313,27 +312,28 @@ __device__ __forceinline__ float group_sum(uint32_t tcol, const float* nc, int n
     float v[32];
     uint64_t ncv[8];
     tmem_ld32(tcol + cc, v);
-    load_nc16(nc + cc, ncv);
+    load_nc16(nc + 4 * cc, ncv);
     tmem_wait_ld();
     if (cc + 32 == ncols) loaded();
     mass_chunk(*reinterpret_cast<float(*)[16]>(v), ncv, al2, a01, a23);
-    load_nc16(nc + cc + 16, ncv);
+    load_nc16(nc + 4 * cc + 64, ncv);
     mass_chunk(*reinterpret_cast<float(*)[16]>(v + 16), ncv, al2, a01, a23);
   }
   if (cc < ncols) {   // an 8-column tail (the anchor rows, r <= 8)
     float v[8];
     tmem_ld8(tcol + cc, v);
-    const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(nc + cc);
-    const ulonglong2 n0 = c2[0], n1 = c2[1];
+    uint64_t n0, n1, n2, n3;
+    lds_2x64(nc + 4 * cc, n0, n1);
+    lds_2x64(nc + 4 * cc + 16, n2, n3);
     tmem_wait_ld();
     loaded();
     float y0, y1, y2, y3;
-    upk2(ffma2(pk2(v[0], v[1]), al2, n0.x), y0, y1);
-    upk2(ffma2(pk2(v[2], v[3]), al2, n0.y), y2, y3);
+    upk2(ffma2(pk2(v[0], v[1]), al2, n0), y0, y1);
+    upk2(ffma2(pk2(v[2], v[3]), al2, n1), y2, y3);
     a01 = fadd2(a01, pk2(fast_exp2(y0), fast_exp2(y1)));
     a23 = fadd2(a23, pk2(fast_exp2(y2), fast_exp2(y3)));
-    upk2(ffma2(pk2(v[4], v[5]), al2, n1.x), y0, y1);
-    upk2(ffma2(pk2(v[6], v[7]), al2, n1.y), y2, y3);
+    upk2(ffma2(pk2(v[4], v[5]), al2, n2), y0, y1);
+    upk2(ffma2(pk2(v[6], v[7]), al2, n3), y2, y3);
     a01 = fadd2(a01, pk2(fast_exp2(y0), fast_exp2(y1)));
     a23 = fadd2(a23, pk2(fast_exp2(y2), fast_exp2(y3)));
   }
@@ -495,7 +495,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     // nothing arrives on, gives up after a few polls and aborts the CTA
     if (P.test_stuck_wait && blockIdx.x == 0 && ew == 0)
       ok = mbar_wait(&never, 0, abort_, kTestSpinLimit);
-    const float* cv = cs_all + ew * SROWS;   // this warp's copy of the block's negated normalisers
+    const uint32_t cv = smem_u32(cs_all + ew * SROWS);   // this warp's copy of the block's negated normalisers
     Block blk{};
     int gb = 0, ge = 0;                      // this warpgroup's groups of the block
     bool my_anchor = false;
@@ -530,7 +530,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         float* out = gdst + kt;
         for (int gi = gb; gi < ge; ++gi, out += P.total_T) {
           const bool last = gi + 1 == ge && !my_anchor;
-          const float sm = group_sum(tacc + (uint32_t)(gi * P.RG), cv + gi * P.RG, P.RG, alpha,
+          const float sm = group_sum(tacc + (uint32_t)(gi * P.RG), cv + 4 * gi * P.RG, P.RG, alpha,
                                      [&] { if (last) release(); });
           if (valid) *out = sm;
         }
@@ -553,7 +553,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           } else {
             // the r anchor rows, in 8-column steps (the padding rows up to 16
             // would add exp2(-inf) = 0)
-            const float sm = group_sum(tacc + (uint32_t)a0, cv + a0, (P.r + 7) & ~7, alpha, release);
+            const float sm = group_sum(tacc + (uint32_t)a0, cv + 4 * a0, (P.r + 7) & ~7, alpha, release);
             if (valid)
               bf.anchor[((size_t)x.l * P.Hkv + x.h) * P.total_T + col] = sm / (float)P.r;
           }
@@ -740,7 +740,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     const int lrow = q * 32 + lane;         // accumulator lane: this CTA's proxy row
     const float alpha = P.alpha;
     const int c_lo = wg * (PBK / 4);
-    const uint32_t tempty_lead[2] = {mapa(smem_u32(&tempty[0]), 0), mapa(smem_u32(&tempty[1]), 0)};
+    const uint32_t tempty_lead = mapa(smem_u32(&tempty[0]), 0);   // the leader's, 8 bytes each
     uint32_t bphase = 0;
     bool ok = true;
     float2* dst = nullptr;
@@ -774,7 +774,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
           if (c0 == PBK / 4 - 32) {
             fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster_relaxed(tempty_lead[buf]);
+            if (lane == 0) mbar_arrive_cluster_relaxed(tempty_lead + 8 * buf);
           }
           if (nvalid < PBK / 4) mask_tail(v, c0, nvalid);   // the last tile of a short split
           if (j == 0 && c0 == 0)

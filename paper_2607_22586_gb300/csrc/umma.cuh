@@ -10,10 +10,14 @@
 namespace mmshift {
 namespace umma {
 
-// Bounded waits: a thread polls an mbarrier at most kSpinLimit times, each
-// poll suspending it for up to kSuspendNs nanoseconds (so waiting threads do
-// not take issue slots from working ones); then it gives up, flags the CTA to
-// abort and lets the kernel report a timeout (about 4 s in the worst case).
+// Bounded waits: a thread first polls an mbarrier kFastPolls times with the
+// plain try_wait, which suspends the thread in hardware for a short while; only
+// a wait that outlasts those polls at most kSpinLimit times more, each poll
+// suspending for up to kSuspendNs nanoseconds; then it gives up, flags the
+// CTA to abort and lets the kernel report a timeout (about 4 s in the worst
+// case). The hinted form costs about ten instructions and a timed sleep per
+// poll, so it stays out of the ordinary path.
+constexpr uint32_t kFastPolls = 64;
 constexpr uint32_t kSpinLimit = 1u << 15;
 constexpr uint32_t kSuspendNs = 100000;
 
@@ -52,16 +56,37 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Wait until the phase of parity `parity` has completed. Returns false if the
-// wait gave up (`limit` polls, or another role already aborted).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
-                                          uint32_t limit = kSpinLimit) {
+__device__ __forceinline__ bool mbar_try_wait_fast(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+// The part of a wait that outlasts the plain polls.
+static __device__ __noinline__ bool mbar_wait_long(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                            uint32_t limit) {
   for (uint32_t i = 0; i < limit; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if (*abort) return false;
   }
   *abort = 1;
   return false;
+}
+
+// Wait until the phase of parity `parity` has completed. Returns false if the
+// wait gave up (after `limit` long polls, or because another role aborted).
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
+                                          uint32_t limit = kSpinLimit) {
+#pragma unroll 1
+  for (uint32_t i = 0; i < kFastPolls; ++i)
+    if (mbar_try_wait_fast(bar, parity)) return true;
+  return mbar_wait_long(bar, parity, abort, limit);
 }
 
 // The same wait without the abort check, for the drain at a CTA's exit: the
@@ -274,6 +299,11 @@ __device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
+}
+
+// Two 64-bit words from a 16-byte aligned shared-memory address.
+__device__ __forceinline__ void lds_2x64(uint32_t saddr, uint64_t& a, uint64_t& b) {
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(saddr));
 }
 
 // Shared-memory matrix descriptor of a K-major operand stored as rows of
