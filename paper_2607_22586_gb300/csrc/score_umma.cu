@@ -343,6 +343,39 @@ __device__ __forceinline__ float group_sum(uint32_t tcol, uint32_t nc, int ncols
   return (a0 + a1) + (a2 + a3);
 }
 
+// The same over NC chunks of 16 columns, unrolled: the tensor-memory load and
+// the normalisers of the next chunk are in flight during the exponentials of
+// the current one. With two draining warps per scheduler the loads of the loop
+// above are exposed: a 112-column sum takes 2,140 clocks there and 1,780 here
+// (448 is the MUFU time of its exponentials), the pass over the 28-layer 32K
+// stack 2.66 and 2.48 ms. Unrolled for the widths of 16 proxies per group under
+// GQA ratios 7 and 8; narrower groups have little to overlap.
+template <int NC, class Loaded>
+__device__ __forceinline__ float group_sum_pipe(uint32_t tcol, uint32_t nc, float alpha,
+                                                const Loaded& loaded) {
+  const uint64_t al2 = pk2(alpha, alpha);
+  uint64_t a01 = 0, a23 = 0;       // (+0, +0)
+  float v[2][16];
+  uint64_t ncv[2][8];
+  tmem_ld16(tcol, v[0]);
+  load_nc16(nc, ncv[0]);
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+    tmem_wait_ld16(v[i & 1]);
+    if (i + 1 < NC) {
+      tmem_ld16(tcol + 16 * (i + 1), v[(i + 1) & 1]);
+      load_nc16(nc + 64 * (i + 1), ncv[(i + 1) & 1]);
+    } else {
+      loaded();
+    }
+    mass_chunk(v[i & 1], ncv[i & 1], al2, a01, a23);
+  }
+  float a0, a1, a2, a3;
+  upk2(a01, a0, a1);
+  upk2(a23, a2, a3);
+  return (a0 + a1) + (a2 + a3);
+}
+
 template <int D, bool LISTS>
 __global__ void __launch_bounds__(NTHREADS, 1)
     mass_umma_kernel(const __grid_constant__ CUtensorMap kmap,
@@ -434,15 +467,20 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    // The whole warp walks the units and one elected lane issues: with uniform
+    // control flow the descriptors stay in uniform registers, which the MMAs
+    // take (a lane-0 branch moves each of them there first).
+    {
       int stage = 0;
       uint32_t phase = 0, bphase = 0, sphase = 0;   // bphase: one phase bit per accumulator
       uint32_t idesc = 0;
+      const uint64_t kd0 = sdesc_k_sw128(smem_u32(ring_buf)), pd0 = sdesc_k_sw128(smem_u32(stat));
       bool ok = true, issued = false;
       while (ok && walk_next<LISTS>(P, S, wk, nwk, x)) {
         if (x.fresh) {
-          if (issued) mma_commit(&sempty);   // old block free once its MMAs finish
-          if (!mbar_wait(&sfull, sphase, abort_)) { ok = false; break; }
+          if (issued && elect_one()) mma_commit(&sempty);   // old block free once its MMAs finish
+          __syncwarp();
+          if (!mbar_wait_warp(&sfull, sphase, abort_)) { ok = false; break; }
           sphase ^= 1u;
           fence_after();
           idesc = idesc_bf16_f32(128, mass_block(P, S, x.tile).rows);
@@ -451,21 +489,22 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         // split's tiles reach the same epilogue warpgroups whatever ran before
         for (int kt = x.t0, j = 0; kt < x.t1; kt += BK, ++j) {
           const int buf = j & 1;
-          if (!mbar_wait(&full[stage], phase, abort_) ||
-              !mbar_wait(&tempty[buf], ((bphase >> buf) & 1u) ^ 1u, abort_)) { ok = false; break; }
+          if (!mbar_wait_warp(&full[stage], phase, abort_) ||
+              !mbar_wait_warp(&tempty[buf], ((bphase >> buf) & 1u) ^ 1u, abort_)) { ok = false; break; }
           fence_after();
-          const uint32_t ks_base = smem_u32(ring_buf + stage * SM::STAGE_BYTES);
-          const uint32_t st_base = smem_u32(stat);
+          const uint64_t kd = kd0 + (uint64_t)(stage * (SM::STAGE_BYTES >> 4));
           const uint32_t dcol = tmem + (uint32_t)(buf * ACC_STRIDE);
+          if (elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) {
-            const int c = ks / 4, w = ks % 4;
-            const uint64_t kd = sdesc_k_sw128(ks_base + c * BK * 128 + w * 32);
-            const uint64_t pd = sdesc_k_sw128(st_base + c * SROWS * 128 + w * 32);
-            mma_bf16(dcol, kd, pd, idesc, ks > 0 ? 1u : 0u);
+            for (int ks = 0; ks < D / 16; ++ks) {
+              const int c = ks / 4, w = ks % 4;
+              mma_bf16(dcol, kd + (uint64_t)((c * BK * 128 + w * 32) >> 4),
+                 pd0 + (uint64_t)((c * SROWS * 128 + w * 32) >> 4), idesc, ks > 0 ? 1u : 0u);
+            }
+            mma_commit(&empty[stage]);
+            mma_commit(&tfull[buf]);
           }
-          mma_commit(&empty[stage]);
-          mma_commit(&tfull[buf]);
+          __syncwarp();
           issued = true;
           if (++stage == NSTAGE) { stage = 0; phase ^= 1u; }
           bphase ^= 1u << buf;
@@ -473,7 +512,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
       // every MMA issued has finished before the CTA's tensor memory goes
       if (issued) {
-        mma_commit(&drain);
+        if (elect_one()) mma_commit(&drain);
+        __syncwarp();
         if (!mbar_wait_drain(&drain, 0)) *abort_ = 1;
       }
     }
@@ -530,8 +570,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         float* out = gdst + kt;
         for (int gi = gb; gi < ge; ++gi, out += P.total_T) {
           const bool last = gi + 1 == ge && !my_anchor;
-          const float sm = group_sum(tacc + (uint32_t)(gi * P.RG), cv + 4 * gi * P.RG, P.RG, alpha,
-                                     [&] { if (last) release(); });
+          auto loaded = [&] { if (last) release(); };
+          const uint32_t tcol = tacc + (uint32_t)(gi * P.RG), nc = cv + 4 * gi * P.RG;
+          float sm;
+          if (P.RG == 112) sm = group_sum_pipe<7>(tcol, nc, alpha, loaded);
+          else if (P.RG == 128) sm = group_sum_pipe<8>(tcol, nc, alpha, loaded);
+          else sm = group_sum(tcol, nc, P.RG, alpha, loaded);
           if (valid) *out = sm;
         }
         if (my_anchor) {
@@ -691,36 +735,39 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
       if (rank == 0 && !(armed_k.drain(full) && armed_s.drain(&sfull))) *abort_ = 1;
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer (leader)
-    if (lane == 0 && rank == 0) {
+    // ------------------------------------------------------------ MMA issuer (leader's warp)
+    if (rank == 0) {
       int stage = 0;
       uint32_t phase = 0, bphase = 0, sphase = 0;
       const uint32_t idesc = idesc_bf16_f32(2 * PROWS, PBK);
+      const uint64_t kd0 = sdesc_k_sw128(smem_u32(ring)), pd0 = sdesc_k_sw128(smem_u32(stat));
       bool ok = true, issued = false;
       while (ok && walk_next<LISTS>(P, S, wk, nwk, x)) {
         if (x.fresh) {
-          if (issued) mma_commit_pair(&sempty, 0x3);   // old block free once its MMAs finish
-          if (!mbar_wait(&sfull, sphase, abort_)) { ok = false; break; }
+          if (issued && elect_one()) mma_commit_pair(&sempty, 0x3);   // old block free once its MMAs finish
+          __syncwarp();
+          if (!mbar_wait_warp(&sfull, sphase, abort_)) { ok = false; break; }
           sphase ^= 1u;
           fence_after();
         }
         for (int kt = x.t0, j = 0; kt < x.t1; kt += PBK, ++j) {
           const int buf = j & 1;
-          if (!mbar_wait(&full[stage], phase, abort_) ||
-              !mbar_wait(&tempty[buf], ((bphase >> buf) & 1u) ^ 1u, abort_)) { ok = false; break; }
+          if (!mbar_wait_warp(&full[stage], phase, abort_) ||
+              !mbar_wait_warp(&tempty[buf], ((bphase >> buf) & 1u) ^ 1u, abort_)) { ok = false; break; }
           fence_after();
-          const uint32_t ks_base = smem_u32(ring + stage * SM::STAGE_BYTES);
-          const uint32_t st_base = smem_u32(stat);
+          const uint64_t kd = kd0 + (uint64_t)(stage * (SM::STAGE_BYTES >> 4));
           const uint32_t dcol = tmem + (uint32_t)(buf * PBK);
+          if (elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < D / 16; ++ks) {
-            const int c = ks / 4, w = ks % 4;
-            mma_bf16_pair(dcol, sdesc_k_sw128(st_base + c * PROWS * 128 + w * 32),
-                          sdesc_k_sw128(ks_base + c * (PBK / 2) * 128 + w * 32), idesc,
-                          ks > 0 ? 1u : 0u);
+            for (int ks = 0; ks < D / 16; ++ks) {
+              const int c = ks / 4, w = ks % 4;
+              mma_bf16_pair(dcol, pd0 + (uint64_t)((c * PROWS * 128 + w * 32) >> 4),
+                 kd + (uint64_t)((c * (PBK / 2) * 128 + w * 32) >> 4), idesc, ks > 0 ? 1u : 0u);
+            }
+            mma_commit_pair(&empty[stage], 0x3);
+            mma_commit_pair(&tfull[buf], 0x3);
           }
-          mma_commit_pair(&empty[stage], 0x3);
-          mma_commit_pair(&tfull[buf], 0x3);
+          __syncwarp();
           issued = true;
           if (++stage == PNSTAGE) { stage = 0; phase ^= 1u; }
           bphase ^= 1u << buf;
@@ -728,7 +775,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
       }
       // every pair MMA issued has finished before either CTA's tensor memory goes
       if (issued) {
-        mma_commit_pair(&drain, 0x1);
+        if (elect_one()) mma_commit_pair(&drain, 0x1);
+        __syncwarp();
         if (!mbar_wait_drain(&drain, 0)) *abort_ = 1;
       }
     }

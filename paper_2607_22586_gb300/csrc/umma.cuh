@@ -89,6 +89,23 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return mbar_wait_long(bar, parity, abort, limit);
 }
 
+// The same wait by a converged warp that stays converged: every lane polls,
+// and all of them leave together with one answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort) {
+#pragma unroll 1
+  for (uint32_t i = 0; i < kFastPolls; ++i)
+    if (__all_sync(0xffffffffu, mbar_try_wait_fast(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait_long(bar, parity, abort, kSpinLimit));
+}
+
+// One lane of a converged warp, always the same one.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok));
+  return ok != 0;
+}
+
 // The same wait without the abort check, for the drain at a CTA's exit: the
 // TMA loads and MMAs a role issued must have finished before the CTA's shared
 // and tensor memory are released, whether or not the CTA aborted.
@@ -200,6 +217,16 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Waits for the warp's tensor-memory loads; v are registers of one of them,
+// named so that no use of them moves above the wait.
+__device__ __forceinline__ void tmem_wait_ld16(float (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]),
+                 "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]),
+                 "+f"(v[13]), "+f"(v[14]), "+f"(v[15])
+               :
+               : "memory");
+}
 __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
