@@ -4,23 +4,34 @@
 // This path serves float32 inputs, for which the tensor cores would round the
 // operands (TF32), and head dims or shapes the tcgen05 path does not cover.
 //
-// Pass 1: CTA = (layer, KV head, key split, 64 packed proxy rows). It streams
-//   the keys of its split through shared memory and keeps, per proxy row, an
-//   online (max, sum of exp2) pair of the log2-scaled logits x = s * alpha,
-//   alpha = softmax_scale * log2(e).
-// Merge: combines the partials of each row (one per key split, two on the
+// Both passes form logits in 64 x 128 tiles (proxy rows x keys) of 128 threads,
+// 8 x 8 per thread, from operands stored transposed in shared memory, so a
+// step of the contraction costs four 16-byte loads per 64 FMAs. Every logit is
+// one chain of FMAs over ascending dimensions.
+// Pass 1: a cluster of up to eight CTAs takes one key split of 64 proxy rows,
+//   each CTA a range of its 128-key tiles; per row and 64 keys a (max, sum of
+//   exp2) pair of the log2-scaled logits x = s * alpha, alpha = softmax_scale
+//   * log2(e), all merged in key order by the cluster's first CTA. Cluster
+//   sizes change who computes a tile, not the result.
+// Merge: combines the partials of each row (one per key split, four on the
 //   tensor-core path) in a fixed order into c = m + log2(Z) (the log2
 //   normaliser), +inf for padding rows so they weigh nothing.
-// Pass 2: CTA = (layer, KV head, 64 keys). It streams every packed proxy row,
-//   recomputes the logits and adds exp2(x - c) into per-(group, key) sums in a
-//   fixed order, then writes the group masses and the anchor (mean over the r
-//   anchor rows).
+// Pass 2: CTA = (layer, KV head, 128 keys, a range of groups). It streams the
+//   groups' proxy rows, recomputes the logits and adds exp2(x - c), 16 rows at
+//   a time in ascending order, into the group masses and the anchor (mean over
+//   the r anchor rows).
+#include <algorithm>
+
 #include "common.cuh"
+#include "umma.cuh"
 
 namespace mmshift {
 namespace {
 
-constexpr int TILE = 64;
+constexpr int TR = 64;      // proxy rows per tile
+constexpr int TK = 128;     // keys per tile: two runs of 64
+constexpr int TNT = 128;    // threads: 8 row groups (8 rows) x 16 key groups (4 + 4 keys)
+constexpr int TRUN = 64;    // keys per (max, sum) pair
 
 __device__ __forceinline__ void find_split(const Problem& P, int s, int& b, int& sl) {
   b = 0;
@@ -28,88 +39,235 @@ __device__ __forceinline__ void find_split(const Problem& P, int s, int& b, int&
   sl = s - P.req[b].split_off;
 }
 
-// 64x64 logits tile: acc[i][j] = A_row(ty*4+i) . B_row(tx*4+j) over D dims,
-// A and B in shared memory with row stride D+1.
-template <int D>
-__device__ __forceinline__ void tile_dot(const float* A, const float* Bm, int ty, int tx,
-                                         float acc[4][4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 4
-  for (int k = 0; k < D; ++k) {
-    float a[4], bv[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) a[i] = A[(ty * 4 + i) * (D + 1) + k];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) bv[j] = Bm[(tx * 4 + j) * (D + 1) + k];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bv[j], acc[i][j]);
+// Four consecutive elements as float32 (`vec`: the pointer allows one load).
+__device__ __forceinline__ float4 load4(const float* p, bool vec) {
+  if (vec) return __ldg(reinterpret_cast<const float4*>(p));
+  return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p, bool vec) {
+  if (vec) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                       __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
   }
+  return make_float4(to_f32(p[0]), to_f32(p[1]), to_f32(p[2]), to_f32(p[3]));
 }
 
+// Shared-memory place of element (row, k) of a transposed tile of R rows
+// (R = 64 or 128). The rows of dimensions 4q..4q+3 are permuted in blocks of
+// eight by q mod 4, which spreads a warp's stores (8 rows x 4 quads) over all
+// banks; a thread still finds its four or eight rows side by side.
+template <int R>
+__device__ __forceinline__ int tile_at(int row, int k) { return k * R + (row ^ (((k >> 2) & 3) << 3)); }
+
+// R rows x KD dimensions of src (rows `stride` elements apart, zeros from row n
+// on), read into registers and stored to a tile in two steps, so that the
+// reads of the next piece are in flight during the FMAs of the current one.
+template <typename T, int R, int KD>
+struct Piece {
+  static constexpr int NB = (R / 8) * (KD / 16) / (TNT / 32);   // 8-row x 16-dimension blocks per warp
+  float4 v[NB];
+  __device__ __forceinline__ static void at(int i, int& row, int& k) {
+    const int e = i * (TNT / 32) + threadIdx.x / 32, lane = threadIdx.x % 32;
+    row = (e / (KD / 16)) * 8 + (lane & 7);
+    k = (e % (KD / 16)) * 16 + (lane >> 3) * 4;
+  }
+  __device__ __forceinline__ void load(const T* src, size_t stride, int n, bool vec) {
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      int row, k;
+      at(i, row, k);
+      v[i] = row < n ? load4(src + (size_t)row * stride + k, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+  __device__ __forceinline__ void store(float* dst) const {
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      int row, k;
+      at(i, row, k);
+      float* d = dst + tile_at<R>(row, k);
+      d[0] = v[i].x;
+      d[R] = v[i].y;
+      d[2 * R] = v[i].z;
+      d[3 * R] = v[i].w;
+    }
+  }
+};
+
+constexpr int KC = 32;      // dimensions per streamed piece
+
+// acc[i][j / 2] += row (ty * 8 + i) . keys (j, j + 1) of the thread over KC
+// dimensions: keys 4 tx .. 4 tx + 3 (j < 4) and 64 + 4 tx .. (j >= 4), in pairs
+// (a packed FMA rounds each half like a scalar one). Bound by FMA issue: 42
+// TFLOP/s on one layer of 4096 keys, d = 128, paper hyper-parameters. With 4 x 4
+// per thread and row-major tiles (two shared-memory loads per four FMAs) that
+// selection took 1398 us, now 803; one layer of 4001 keys with 1,024 packed
+// rows per KV head 398 -> 290 us, one layer of 1024 keys, d = 64, 294 -> 101 us
+// (36 and 16 CTAs before, 264 and 272 now). Scalar FMAs take 331 us on the second.
+__device__ __forceinline__ void tile_dot(const float* As, const float* Bs, int ty, int tx,
+                                         uint64_t (&acc)[8][4]) {
+#pragma unroll 1
+  for (int k0 = 0; k0 < KC; k0 += 16) {
+#pragma unroll
+    for (int kk = 0; kk < 16; ++kk) {
+      const int x = (kk >> 2) << 3;            // tile_at's permutation of dimension k0 + kk
+      const float* ap = As + (k0 + kk) * TR + ((ty * 8) ^ x);
+      const float* bp = Bs + (k0 + kk) * TK + ((tx * 4) ^ x);
+      const float4 a0 = *reinterpret_cast<const float4*>(ap);
+      const float4 a1 = *reinterpret_cast<const float4*>(ap + 4);
+      const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(bp);
+      const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(bp + TRUN);
+      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const uint64_t b[4] = {b0.x, b0.y, b1.x, b1.y};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint64_t aa = umma::pk2(a[i], a[i]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = umma::ffma2(aa, b[j], acc[i][j]);
+      }
+    }
+  }
+}
+__device__ __forceinline__ void clear(uint64_t (&acc)[8][4]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0;     // (+0, +0)
+}
+// Logit j (0-7) of row i.
+__device__ __forceinline__ float logit(const uint64_t (&acc)[8][4], int i, int j) {
+  float lo, hi;
+  umma::upk2(acc[i][j >> 1], lo, hi);
+  return (j & 1) ? hi : lo;
+}
+
+// Shared::cluster address of this CTA's shared-memory location in CTA `rank`,
+// and a 64-bit load from there.
+__device__ __forceinline__ float2 ld_cluster_f2(const float2* p, int rank) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  uint32_t c;
+  float2 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(c) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(c) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 template <typename T, int D>
-__global__ void __launch_bounds__(256) pass1_simt(Problem P, Buffers bf, const T* K) {
+__global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Problem P, Buffers bf,
+                                                  const T* K, int nrank, bool vec) {
   extern __shared__ float sm[];
-  float* Ps = sm;                    // [64][D+1] proxy rows
-  float* Ks = Ps + TILE * (D + 1);   // [64][D+1] keys
-  float* Ls = Ks + TILE * (D + 1);   // [64][65] scaled logits
-  const int n_rt = P.Prows_pad / TILE;
+  float* As = sm;                    // [D][64] proxy rows
+  float* Bs = As + TR * D;           // [2][KC][128] keys, a piece and the next one
+  float2* pairs = reinterpret_cast<float2*>(Bs + 2 * KC * TK);   // [runs of this CTA][64] (max, sum)
+  const int n_rt = (P.Prows + TR - 1) / TR;
   int u = blockIdx.x;
+  const int rank = u % nrank; u /= nrank;
   const int rt = u % n_rt; u /= n_rt;
   const int s = u % P.total_splits; u /= P.total_splits;
   const int h = u, l = blockIdx.y;
   int b, sl;
   find_split(P, s, b, sl);
-  const ReqInfo R = P.req[b];
-  const int t0 = sl * P.split_len, t1 = min(R.t_len, t0 + P.split_len);
+  const int t_len = P.req[b].t_len, tok_off = P.req[b].tok_off;
+  const int t0 = sl * P.split_len, t1 = min(t_len, t0 + P.split_len);
   const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
+  // this CTA's tiles of the split: rank r takes tiles [r, r + 1) * ntiles / nrank
+  const int ntiles = (t1 - t0 + TK - 1) / TK;
+  const int k0 = rank * ntiles / nrank, k1 = (rank + 1) * ntiles / nrank;
 
   const T* pk = (const T*)bf.packed +
-                ((((size_t)l * P.B + b) * P.Hkv + h) * P.Prows_pad + (size_t)rt * TILE) * D;
-  for (int e = tid; e < TILE * D; e += 256) Ps[(e / D) * (D + 1) + e % D] = to_f32(pk[e]);
-  const T* kb = K + (size_t)l * P.ls_kv + ((size_t)R.tok_off * P.Hkv + h) * D;
+                ((((size_t)l * P.B + b) * P.Hkv + h) * P.Prows_pad + (size_t)rt * TR) * D;
   const size_t kstride = (size_t)P.Hkv * D;
-
-  float run_m = -INFINITY, run_z = 0.f;
-  const int row = tid / 4, part = tid % 4;
-  for (int kt = t0; kt < t1; kt += TILE) {
-    __syncthreads();
-    for (int e = tid; e < TILE * D; e += 256) {
-      const int kk = e / D, c = e - kk * D, t = kt + kk;
-      Ks[kk * (D + 1) + c] = t < t1 ? to_f32(kb[(size_t)t * kstride + c]) : 0.f;
+  const T* kb = K + (size_t)l * P.ls_kv + (size_t)tok_off * kstride + (size_t)h * D;
+  // pieces of KC dimensions of the CTA's tiles, one after the other
+  constexpr int NP = D / KC;
+  const int np = (k1 - k0) * NP;
+  Piece<T, TK, KC> next;
+  auto fetch = [&](int p) {
+    const int tk = t0 + (k0 + p / NP) * TK;
+    next.load(kb + (size_t)tk * kstride + (p % NP) * KC, kstride, t1 - tk, vec);
+  };
+  if (np) {
+    fetch(0);
+#pragma unroll 1
+    for (int c = 0; c < NP; ++c) {              // Prows_pad is a multiple of TR
+      Piece<T, TR, KC> a;
+      a.load(pk + c * KC, D, TR, true);
+      a.store(As + c * KC * TR);
     }
-    __syncthreads();
-    float acc[4][4];
-    tile_dot<D>(Ps, Ks, ty, tx, acc);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int kk = tx * 4 + j;
-        Ls[(ty * 4 + i) * (TILE + 1) + kk] = (kt + kk < t1) ? acc[i][j] * P.alpha : -INFINITY;
-      }
-    __syncthreads();
-    float m = -INFINITY;
-    for (int c = part * 16; c < part * 16 + 16; ++c) m = fmaxf(m, Ls[row * (TILE + 1) + c]);
-    float z = 0.f;
-    if (m != -INFINITY)
-      for (int c = part * 16; c < part * 16 + 16; ++c) z += fast_exp2(Ls[row * (TILE + 1) + c] - m);
-#pragma unroll
-    for (int off = 1; off < 4; off <<= 1) {
-      const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
-      const float z2 = __shfl_xor_sync(0xffffffffu, z, off);
-      merge_ms(m, z, m2, z2);
-    }
-    merge_ms(run_m, run_z, m, z);
+    next.store(Bs);
   }
-  if (part == 0)
+  __syncthreads();
+  uint64_t acc[8][4];
+#pragma unroll 1
+  for (int p = 0; p < np; ++p) {
+    const int c = p % NP, kt = k0 + p / NP, tk = t0 + kt * TK;
+    if (p + 1 < np) fetch(p + 1);
+    if (c == 0) clear(acc);
+    tile_dot(As + c * KC * TR, Bs + (p & 1) * KC * TK, ty, tx, acc);
+    if (p + 1 < np) next.store(Bs + ((p + 1) & 1) * KC * TK);
+    __syncthreads();
+    if (c != NP - 1) continue;
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        // 16 keys are the four keys of four lanes in a row: their max, then
+        // their sum as one chain over ascending keys
+        float x[4], m = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          x[j] = tk + half * TRUN + tx * 4 + j < t1 ? logit(acc, i, half * 4 + j) * P.alpha : -INFINITY;
+          m = fmaxf(m, x[j]);
+        }
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        float z = 0.f;
+        if (m != -INFINITY) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[j] = fast_exp2(x[j] - m);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[j] = 0.f;
+        }
+#pragma unroll
+        for (int step = 0; step < 4; ++step) {
+          const float zin = __shfl_up_sync(0xffffffffu, z, 1);
+          if ((tx & 3) == step) {
+            z = step ? zin : 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) z += x[j];
+          }
+        }
+        z = __shfl_sync(0xffffffffu, z, (tid & 28) | 3);
+        // the run's four 16-key pairs, two by two
+#pragma unroll
+        for (int off = 4; off < 16; off <<= 1) {
+          const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
+          const float z2 = __shfl_xor_sync(0xffffffffu, z, off);
+          merge_ms(m, z, m2, z2);
+        }
+        if (tx == 0) pairs[(size_t)((kt - k0) * 2 + half) * TR + ty * 8 + i] = make_float2(m, z);
+      }
+    }
+  }
+  if (nrank > 1) cluster_barrier(); else __syncthreads();
+  if (rank == 0 && tid < TR && rt * TR + tid < P.Prows_pad) {
+    float run_m = -INFINITY, run_z = 0.f;
+    for (int r = 0; r < nrank; ++r) {
+      const int n = 2 * ((r + 1) * ntiles / nrank - r * ntiles / nrank);
+      for (int i = 0; i < n; ++i) {
+        const float2* p = pairs + (size_t)i * TR + tid;
+        const float2 v = r == 0 ? *p : ld_cluster_f2(p, r);
+        merge_ms(run_m, run_z, v.x, v.y);
+      }
+    }
     bf.part[(((size_t)l * P.Hkv + h) * P.total_splits + s) * P.part_slots * P.Prows_pad +
-            rt * TILE + row] = make_float2(run_m, run_z);
+            rt * TR + tid] = make_float2(run_m, run_z);
+  }
+  if (nrank > 1) cluster_barrier();   // no CTA leaves while the first may still read its pairs
 }
 
 // SUB threads per row (four when a row has at least 128 partials, else one):
@@ -157,92 +315,166 @@ __global__ void merge_kernel(Problem P, Buffers bf) {
 }
 
 template <typename T, int D>
-__global__ void __launch_bounds__(256) pass2_simt(Problem P, Buffers bf, const T* K) {
+__global__ void __launch_bounds__(TNT, 2) pass2_simt(const __grid_constant__ Problem P, Buffers bf,
+                                                  const T* K, int gper, bool vec) {
   extern __shared__ float sm[];
-  float* Ks = sm;                    // [64][D+1] keys (stationary)
-  float* Ps = Ks + TILE * (D + 1);   // [64][D+1] proxy rows
-  float* Ls = Ps + TILE * (D + 1);   // [64][65] exp2(x - c)
-  float* cs = Ls + TILE * (TILE + 1);// [64]
-  float* gacc = cs + TILE;           // [G+1][64]
+  float* Bs = sm;                    // [D][128] keys (stationary)
+  float* As = Bs + TK * D;           // [2][KC][64] proxy rows, a piece and the next one
+  float* sums = As + 2 * KC * TR;    // [4][128] sums over 16 rows
+  const int ngr = (P.G + 1 + gper - 1) / gper;   // group ranges; the anchor is group G
   int u = blockIdx.x;
   const int l = blockIdx.y;
+  const int g0 = (u % ngr) * gper, g1 = min(P.G + 1, g0 + gper);
+  u /= ngr;
   const int h = u % P.Hkv;
   u /= P.Hkv;
   int b = 0;
   for (; b < P.B; ++b) {
-    const int nt = (P.req[b].t_len + TILE - 1) / TILE;
+    const int nt = (P.req[b].t_len + TK - 1) / TK;
     if (u < nt) break;
     u -= nt;
   }
-  const ReqInfo R = P.req[b];
-  const int kt = u * TILE;
-  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
-  const T* kb = K + (size_t)l * P.ls_kv + ((size_t)R.tok_off * P.Hkv + h) * D;
+  const int t_len = P.req[b].t_len, tok_off = P.req[b].tok_off;
+  const int kt = u * TK;
+  const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16, lane = tid % 32, w = tid / 32;
   const size_t kstride = (size_t)P.Hkv * D;
-  for (int e = tid; e < TILE * D; e += 256) {
-    const int kk = e / D, c = e - kk * D, t = kt + kk;
-    Ks[kk * (D + 1) + c] = t < R.t_len ? to_f32(kb[(size_t)t * kstride + c]) : 0.f;
-  }
-  for (int e = tid; e < (P.G + 1) * TILE; e += 256) gacc[e] = 0.f;
+  const T* kb = K + (size_t)l * P.ls_kv + ((size_t)tok_off + kt) * kstride + (size_t)h * D;
   const T* pk = (const T*)bf.packed + ((((size_t)l * P.B + b) * P.Hkv + h) * P.Prows_pad) * D;
   const float* cv = bf.cvals + (((size_t)l * P.B + b) * P.Hkv + h) * P.Prows_pad;
-  const int key = tid % TILE, ch = tid / TILE;
-  for (int pt = 0; pt < P.Prows_pad / TILE; ++pt) {
-    __syncthreads();
-    for (int e = tid; e < TILE * D; e += 256)
-      Ps[(e / D) * (D + 1) + e % D] = to_f32(pk[(size_t)pt * TILE * D + e]);
-    if (tid < TILE) cs[tid] = cv[pt * TILE + tid];
-    __syncthreads();
-    float acc[4][4];
-    tile_dot<D>(Ps, Ks, ty, tx, acc);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int pr = ty * 4 + i;
-        Ls[pr * (TILE + 1) + tx * 4 + j] = fast_exp2(fmaf(acc[i][j], P.alpha, -cs[pr]));
-      }
-    __syncthreads();
-    float csum = 0.f;
-    for (int rr = 0; rr < kChunk; ++rr) csum += Ls[(ch * kChunk + rr) * (TILE + 1) + key];
-    const int g = chunk_group(P, pt * (TILE / kChunk) + ch);
-    for (int c = 0; c < TILE / kChunk; ++c) {
-      if (ch == c) gacc[g * TILE + key] += csum;
-      __syncthreads();
+  // 16-row chunks of the groups g0 .. g1 - 1
+  const int c_lo = g0 * (P.RG / kChunk);
+  const int c_hi = g1 <= P.G ? g1 * (P.RG / kChunk) : P.Prows / kChunk;
+  const int t = kt + tid;            // the key whose masses this thread adds up
+  int cur = g0;
+  float gsum = 0.f;
+  auto flush = [&] {
+    if (t < t_len) {
+      const size_t col = (size_t)tok_off + t;
+      if (cur < P.G) bf.gmass[(((size_t)l * P.Hkv + h) * P.G + cur) * P.total_T + col] = gsum;
+      else bf.anchor[((size_t)l * P.Hkv + h) * P.total_T + col] = gsum / (float)P.r;
     }
+    gsum = 0.f;
+  };
+  // pieces of KC dimensions of the 64-row tiles, one after the other
+  constexpr int NP = D / KC, CPT = TR / kChunk;
+  const int np = (c_hi - c_lo + CPT - 1) / CPT * NP;
+  Piece<T, TR, KC> next;
+  auto fetch = [&](int p) {
+    const int row0 = (c_lo + p / NP * CPT) * kChunk;
+    next.load(pk + (size_t)row0 * D + (p % NP) * KC, D, P.Prows_pad - row0, true);
+  };
+  fetch(0);
+#pragma unroll 1
+  for (int c = 0; c < NP; ++c) {
+    Piece<T, TK, KC> k;
+    k.load(kb + c * KC, kstride, t_len - kt, vec);
+    k.store(Bs + c * KC * TK);
   }
+  next.store(As);
   __syncthreads();
-  const int t = kt + key;
-  if (t < R.t_len) {
-    const size_t col = (size_t)R.tok_off + t;
-    for (int g = ch; g < P.G; g += 256 / TILE)
-      bf.gmass[(((size_t)l * P.Hkv + h) * P.G + g) * P.total_T + col] = gacc[g * TILE + key];
-    if (ch == 0)
-      bf.anchor[((size_t)l * P.Hkv + h) * P.total_T + col] = gacc[P.G * TILE + key] / (float)P.r;
+  uint64_t acc[8][4];
+  float cn[8];            // cn: normalisers of the thread's eight rows
+#pragma unroll 1
+  for (int p = 0; p < np; ++p) {
+    const int pc = p % NP, c0 = c_lo + p / NP * CPT;
+    if (p + 1 < np) fetch(p + 1);
+    if (pc == 0) {
+      clear(acc);
+      const int row = c0 * kChunk + ty * 8;     // rows in eights: all or none inside
+#pragma unroll
+      for (int i = 0; i < 8; ++i) cn[i] = row < P.Prows_pad ? __ldg(cv + row + i) : INFINITY;
+    }
+    tile_dot(As + (p & 1) * KC * TR, Bs + pc * KC * TK, ty, tx, acc);
+    if (p + 1 < np) next.store(As + ((p + 1) & 1) * KC * TR);
+    if (pc != NP - 1) {
+      __syncthreads();
+      continue;
+    }
+    // per key, the 16 rows of a chunk (two threads: lanes i and i + 16) as one
+    // chain over ascending rows
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float e[8], z = 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) e[i] = fast_exp2(fmaf(logit(acc, i, j), P.alpha, -cn[i]));
+      if (lane < 16) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) z += e[i];
+      }
+      z = __shfl_sync(0xffffffffu, z, lane & 15);
+      if (lane >= 16) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) z += e[i];
+        sums[w * TK + (j < 4 ? 0 : TRUN) + tx * 4 + (j & 3)] = z;
+      }
+    }
+    __syncthreads();
+    for (int c = 0; c < CPT && c0 + c < c_hi; ++c) {
+      const int g = chunk_group(P, c0 + c);
+      if (g != cur) { flush(); cur = g; }
+      gsum += sums[c * TK + tid];
+    }
+    __syncthreads();   // the sums are read before the next tile's are written
   }
+  flush();
 }
 
 template <typename T, int D>
 cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K,
                      cudaEvent_t* ev) {
-  const size_t sm1 = (2 * TILE * (D + 1) + TILE * (TILE + 1)) * sizeof(float);
-  const size_t sm2 = sm1 + (TILE + (size_t)(P.G + 1) * TILE) * sizeof(float);
   cudaError_t e;
+  int dev = 0, nsm = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  // four elements of a row in one load: K's base, rows and layers allow it
+  const size_t quad = 4 * sizeof(T);
+  const bool vec = reinterpret_cast<uintptr_t>(K) % quad == 0 && (P.ls_kv * sizeof(T)) % quad == 0;
+  // pass 1: more CTAs per split (a cluster), up to one per 128-key tile, until
+  // each SM has its three CTAs: more of them read the proxy rows once more
+  // each (4 rounds: 344 us against 331 on 4001 keys, 930 against 899 at 4096 keys
+  // with paper hyper-parameters), fewer leave SMs idle on short calls
+  const int n_rt = (P.Prows + TR - 1) / TR;
+  int max_len = 1;
+  for (int b = 0; b < P.B; ++b) max_len = std::max(max_len, std::min(P.req[b].t_len, P.split_len));
+  const int max_tiles = (max_len + TK - 1) / TK;
+  const long long units = (long long)P.Hkv * P.total_splits * n_rt * P.L;
+  int nrank = 1;
+  while (nrank < 8 && nrank < max_tiles && units * nrank < 3LL * nsm) nrank *= 2;
+  const int runs = 2 * ((max_tiles + nrank - 1) / nrank);
+  const size_t sm1 = (size_t)(TR * D + 2 * KC * TK) * sizeof(float) + (size_t)runs * TR * sizeof(float2);
   if ((e = cudaFuncSetAttribute(pass1_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sm1)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(pass2_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)sm2)) != cudaSuccess) return e;
-  dim3 g1(P.Hkv * P.total_splits * (P.Prows_pad / TILE), P.L);
   if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
-  pass1_simt<T, D><<<g1, 256, sm1, st>>>(P, bf, (const T*)K);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(P.Hkv * P.total_splits * n_rt * nrank), P.L);
+  cfg.blockDim = dim3(TNT);
+  cfg.dynamicSmemBytes = sm1;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = nrank;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if ((e = cudaLaunchKernelEx(&cfg, pass1_simt<T, D>, P, bf, (const T*)K, nrank, vec)) != cudaSuccess)
+    return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   if ((e = launch_merge(P, bf, st)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
-  int tiles = 0;
-  for (int b = 0; b < P.B; ++b) tiles += (P.req[b].t_len + TILE - 1) / TILE;
-  dim3 g2(P.Hkv * tiles, P.L);
-  pass2_simt<T, D><<<g2, 256, sm2, st>>>(P, bf, (const T*)K);
+  // pass 2: whole groups spread over CTAs, about three rounds of the two an SM
+  // takes (the key tile is loaded once per CTA: two rounds 334 us, eight 343)
+  long long tiles = 0;
+  for (int b = 0; b < P.B; ++b) tiles += (P.req[b].t_len + TK - 1) / TK;
+  const long long keyu = tiles * P.Hkv * P.L;
+  const int want = (int)std::min<long long>(P.G + 1, std::max<long long>(1, (6LL * nsm + keyu - 1) / keyu));
+  const int gper = (P.G + 1 + want - 1) / want;
+  const int ngr = (P.G + 1 + gper - 1) / gper;
+  const size_t sm2 = (size_t)(TK * D + 2 * KC * TR + 4 * TK) * sizeof(float);
+  if ((e = cudaFuncSetAttribute(pass2_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sm2)) != cudaSuccess) return e;
+  pass2_simt<T, D><<<dim3((unsigned)(tiles * P.Hkv * ngr), P.L), TNT, sm2, st>>>(P, bf, (const T*)K,
+                                                                              gper, vec);
   return cudaGetLastError();
 }
 
