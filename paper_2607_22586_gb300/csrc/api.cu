@@ -678,6 +678,73 @@ static mmshift_status coverage_params(int32_t n_dec, float softmax_scale, mmshif
   return MMSHIFT_OK;
 }
 
+// The two-softmax form of the coverage: the decode queries of a KV head's r
+// query heads as one group of proxies without anchor rows, over the prompt (P)
+// and over the kept rows (Pk: the output layout as a varlen batch of its own).
+struct CoverageJob {
+  Problem P, Pk;
+  size_t packed, part, part_k, kept, kept_len, total;   // workspace offsets (status word first)
+};
+
+static void coverage_job(const Problem& steps, CoverageJob* J) {
+  Problem& P = J->P;
+  P = steps;
+  P.G = 1;
+  P.gs = P.Np;
+  P.RG = roundup(P.r * P.gs, kChunk);
+  P.n_group_rows = P.Prows = P.RG;
+  P.anchor_rows = 0;
+  P.Prows_pad = roundup(P.Prows, kRowTile);
+  P.anchor_split = 0;
+  Problem& Q = J->Pk;
+  Q = P;
+  Q.total_T = P.R;
+  Q.ls_kv = P.L > 1 ? (int64_t)P.R * P.Hkv * P.d : 0;
+  int32_t so = 0;
+  for (int b = 0; b < P.B; ++b) {
+    ReqInfo& R = Q.req[b];
+    R.t_len = R.keep;
+    R.tok_off = R.out_off;
+    R.nsplit = (R.t_len + Q.split_len - 1) / Q.split_len;
+    R.split_off = so;
+    so += R.nsplit;
+  }
+  Q.total_splits = so;
+  const size_t esz = P.dtype == MMSHIFT_BF16 ? 2 : 4, L = P.L;
+  size_t o = 256;
+  J->packed = o;   o += align256(L * P.B * P.Hkv * (size_t)P.Prows_pad * P.d * esz);
+  J->part = o;     o += align256(L * P.Hkv * (size_t)P.total_splits * kUmmaPartSlots * P.Prows_pad * sizeof(float2));
+  J->part_k = o;   o += align256(L * P.Hkv * (size_t)Q.total_splits * kUmmaPartSlots * P.Prows_pad * sizeof(float2));
+  J->kept = o;     o += align256(L * (size_t)P.R * P.Hkv * P.d * esz);
+  J->kept_len = o; o += align256(L * P.B * P.Hkv * sizeof(int32_t));
+  J->total = o;
+}
+
+static mmshift_status run_coverage(CoverageJob& J, const void* K, const void* dec_q,
+                                   const int32_t* idx, float* cov, char* ws, cudaStream_t st) {
+  Problem &P = J.P, &Q = J.Pk;
+  P.use_umma = Q.use_umma =
+      umma_softmax_supported(P) && (reinterpret_cast<uintptr_t>(K) & 15) == 0 ? 1 : 0;
+  P.part_slots = Q.part_slots = P.use_umma ? kUmmaPartSlots : 1;
+  Buffers bf;
+  std::memset(&bf, 0, sizeof(bf));
+  bf.status = reinterpret_cast<int*>(ws);
+  bf.packed = ws + J.packed;
+  bf.part = reinterpret_cast<float2*>(ws + J.part);
+  bf.proxies_in = dec_q;
+  Buffers bk = bf;
+  bk.part = reinterpret_cast<float2*>(ws + J.part_k);
+  int32_t* klen = reinterpret_cast<int32_t*>(ws + J.kept_len);
+  bk.kept_len = klen;
+  void* kept = ws + J.kept;
+  cudaError_t e = launch_proxy_pack(P, bf, st, nullptr);
+  if (e == cudaSuccess) e = launch_kept_rows(P, K, idx, kept, klen, bf.status, st);
+  if (e == cudaSuccess) e = P.use_umma ? launch_softmax_umma(P, bf, st, K) : launch_softmax_simt(P, bf, st, K);
+  if (e == cudaSuccess) e = Q.use_umma ? launch_softmax_umma(Q, bk, st, kept) : launch_softmax_simt(Q, bk, st, kept);
+  if (e == cudaSuccess) e = launch_coverage_ratio(P, Q, bf.part, bk.part, cov, st);
+  return e == cudaSuccess ? MMSHIFT_OK : cuda_fail(e);
+}
+
 mmshift_status mmshift_coverage_workspace_size(const mmshift_shape* s, int32_t n_dec,
                                                size_t* bytes) {
   mmshift_params p;
@@ -699,9 +766,16 @@ mmshift_status mmshift_coverage(const mmshift_shape* s, const void* K, const voi
   set_score_path(P, K);
   Buffers bf;
   if ((st = carve(P, workspace, workspace_bytes, &bf)) != MMSHIFT_OK) return st;
+  const cudaStream_t cs = (cudaStream_t)stream;
+  // two softmax passes where the copied kept rows fit in the workspace that
+  // steps 2-4 need (its size is the entry's contract either way): with 32
+  // decode queries, budgets up to about half the prompt
+  CoverageJob J;
+  coverage_job(P, &J);
+  if (J.total <= layout_of(P).total)
+    return run_coverage(J, K, dec_q, idx, cov, static_cast<char*>(workspace), cs);
   bf.proxies_in = dec_q;
   bf.mass = nullptr;
-  const cudaStream_t cs = (cudaStream_t)stream;
   if ((st = run_mass(P, bf, K, Qwin, cs)) != MMSHIFT_OK) return st;
   const cudaError_t e = launch_coverage(P, bf, idx, cov, cs);
   return e == cudaSuccess ? MMSHIFT_OK : cuda_fail(e);

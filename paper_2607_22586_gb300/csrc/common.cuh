@@ -86,6 +86,9 @@ struct Buffers {
   const float* stats_in;  // [L][B][2][Hq][d] mean / std of the proxies, or null (window's)
   const int32_t* head_budget; // [L][B][Hkv] budgets C_{l,b,h} in [1, C_b], or null (C_b for all)
   int32_t* out_count;         // [L][B][Hkv] kept rows per head, or null
+  // keys of each (layer, request, KV head) that the softmax pass takes, or
+  // null (all T_b): the kept rows of a coverage call
+  const int32_t* kept_len;    // [L][B][Hkv]
   // bf16 proxies whose float32 value lies too close to a rounding boundary
   // are recomputed in float64 (proxy.cu): the sampler appends them here and a
   // second kernel redoes them; without a list (null) the sampler redoes them
@@ -194,6 +197,12 @@ cudaError_t launch_score_simt(const Problem& P, const Buffers& bf, cudaStream_t 
 cudaError_t launch_score_umma(const Problem& P, const Buffers& bf, cudaStream_t st,
                               const void* K, cudaEvent_t* ev);
 bool umma_supported(const Problem& P);
+// The softmax pass alone (partials in bf.part), for sums whose ratio is the
+// result: on the tensor cores where umma_softmax_supported says so, else on the
+// CUDA cores.
+bool umma_softmax_supported(const Problem& P);
+cudaError_t launch_softmax_umma(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K);
+cudaError_t launch_softmax_simt(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K);
 // Scratch of launch_hidden_proxies (sampled hidden states, RoPE table) and
 // the launch itself: sampling kernel, then the projection GEMM.
 size_t hidden_scratch_bytes(const HiddenJob& J);
@@ -208,6 +217,16 @@ bool tmap_encoder_available();
 int umma_launches(const Problem& P);
 cudaError_t launch_anchor_split(const Problem& P, const Buffers& bf, cudaStream_t st);
 cudaError_t launch_merge(const Problem& P, const Buffers& bf, cudaStream_t st);
+// Copies the kept rows of K (idx; -1 and bad indices left out, the bad ones
+// reported) to kept [L][R][Hkv][d], each (layer, request, KV head)'s rows
+// together from its first output row on, and their number to kept_len.
+cudaError_t launch_kept_rows(const Problem& P, const void* K, const int32_t* idx, void* kept,
+                             int32_t* kept_len, int* status, cudaStream_t st);
+// cov = mean over the query heads of (sum over the kept keys) / (sum over all
+// keys) of each decode query's exponentials, from the two softmax passes'
+// partials: `all` over the prompt (problem P), `kept` over the kept rows (Pk).
+cudaError_t launch_coverage_ratio(const Problem& P, const Problem& Pk, const float2* all,
+                                  const float2* kept, float* cov, cudaStream_t st);
 // Attention-mass coverage of the kept set idx from the group masses in bf.
 cudaError_t launch_coverage(const Problem& P, const Buffers& bf, const int32_t* idx, float* cov,
                             cudaStream_t st);

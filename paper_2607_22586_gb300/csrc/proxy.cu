@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
       sg[k] = st[(size_t)P.Hq * D + k];
       mmag[k] = fabsf(mu[k]);
     }
-  } else {
+  } else if (!bf.proxies_in) {
     // exact window sums: thread (k, rg) takes rows rg, rg + RPT, ... of
     // dimension k (independent, unrolled loads); the block adds the partials
     const int k = threadIdx.x % D, rg = threadIdx.x / D;
@@ -369,13 +369,15 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
   }
   if (!packed || chunk != 0) return;
   // anchor row of this query head: the last window query as given
-  T* arow = packed + (size_t)(P.n_group_rows + j) * D;
-  for (int k = threadIdx.x; k < D; k += blockDim.x) arow[k] = q[(size_t)(P.W - 1) * qstride + k];
+  if (P.anchor_rows) {
+    T* arow = packed + (size_t)(P.n_group_rows + j) * D;
+    for (int k = threadIdx.x; k < D; k += blockDim.x) arow[k] = q[(size_t)(P.W - 1) * qstride + k];
+  }
   // padding rows (the tail of each group's rows, of the anchor rows and of
   // the block) are zeroed by the first query head of the KV head
   if (j == 0) {
     const int gpad = P.RG - P.r * P.gs;                  // per group
-    const int apad = P.anchor_rows - P.r;                // after the anchor rows
+    const int apad = P.anchor_rows ? P.anchor_rows - P.r : 0;   // after the anchor rows
     const int tail = P.Prows_pad - P.Prows;              // after the last block row
     const int n_pad = P.G * gpad + apad + tail;
     for (int e = threadIdx.x; e < n_pad * D; e += blockDim.x) {

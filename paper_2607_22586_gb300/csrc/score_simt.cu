@@ -171,10 +171,12 @@ __global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Pro
   int b, sl;
   find_split(P, s, b, sl);
   const int t_len = P.req[b].t_len, tok_off = P.req[b].tok_off;
-  const int t0 = sl * P.split_len, t1 = min(t_len, t0 + P.split_len);
+  const int t0 = sl * P.split_len;
+  int t1 = min(t_len, t0 + P.split_len);
+  if (bf.kept_len) t1 = min(t1, bf.kept_len[((size_t)l * P.B + b) * P.Hkv + h]);
   const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
   // this CTA's tiles of the split: rank r takes tiles [r, r + 1) * ntiles / nrank
-  const int ntiles = (t1 - t0 + TK - 1) / TK;
+  const int ntiles = max(0, t1 - t0 + TK - 1) / TK;
   const int k0 = rank * ntiles / nrank, k1 = (rank + 1) * ntiles / nrank;
 
   const T* pk = (const T*)bf.packed +
@@ -419,16 +421,25 @@ __global__ void __launch_bounds__(TNT, 2) pass2_simt(const __grid_constant__ Pro
   flush();
 }
 
-template <typename T, int D>
-cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K,
-                     cudaEvent_t* ev) {
-  cudaError_t e;
-  int dev = 0, nsm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  // four elements of a row in one load: K's base, rows and layers allow it
+cudaError_t device_sms(int* nsm) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e : cudaDeviceGetAttribute(nsm, cudaDevAttrMultiProcessorCount, dev);
+}
+
+// Four elements of a row in one load: K's base, rows and layers allow it.
+template <typename T>
+bool quad_loads(const Problem& P, const void* K) {
   const size_t quad = 4 * sizeof(T);
-  const bool vec = reinterpret_cast<uintptr_t>(K) % quad == 0 && (P.ls_kv * sizeof(T)) % quad == 0;
+  return reinterpret_cast<uintptr_t>(K) % quad == 0 && (P.ls_kv * sizeof(T)) % quad == 0;
+}
+
+template <typename T, int D>
+cudaError_t launch_pass1(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K) {
+  int nsm = 0;
+  cudaError_t e = device_sms(&nsm);
+  if (e != cudaSuccess) return e;
+  const bool vec = quad_loads<T>(P, K);
   // pass 1: more CTAs per split (a cluster), up to one per 128-key tile, until
   // each SM has its three CTAs: more of them read the proxy rows once more
   // each (4 rounds: 344 us against 331 on 4001 keys, 930 against 899 at 4096 keys
@@ -444,7 +455,6 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
   const size_t sm1 = (size_t)(TR * D + 2 * KC * TK) * sizeof(float) + (size_t)runs * TR * sizeof(float2);
   if ((e = cudaFuncSetAttribute(pass1_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sm1)) != cudaSuccess) return e;
-  if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(P.Hkv * P.total_splits * n_rt * nrank), P.L);
   cfg.blockDim = dim3(TNT);
@@ -457,8 +467,18 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if ((e = cudaLaunchKernelEx(&cfg, pass1_simt<T, D>, P, bf, (const T*)K, nrank, vec)) != cudaSuccess)
-    return e;
+  return cudaLaunchKernelEx(&cfg, pass1_simt<T, D>, P, bf, (const T*)K, nrank, vec);
+}
+
+template <typename T, int D>
+cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K,
+                     cudaEvent_t* ev) {
+  int nsm = 0;
+  cudaError_t e = device_sms(&nsm);
+  if (e != cudaSuccess) return e;
+  const bool vec = quad_loads<T>(P, K);
+  if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
+  if ((e = launch_pass1<T, D>(P, bf, st, K)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   if ((e = launch_merge(P, bf, st)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
@@ -494,6 +514,14 @@ cudaError_t launch_merge(const Problem& P, const Buffers& bf, cudaStream_t st) {
     merge_kernel<1><<<grid, threads, 0, st>>>(P, bf);
   }
   return cudaGetLastError();
+}
+
+cudaError_t launch_softmax_simt(const Problem& P, const Buffers& bf, cudaStream_t st,
+                                const void* K) {
+  if (P.dtype == MMSHIFT_BF16)
+    return P.d == 128 ? launch_pass1<__nv_bfloat16, 128>(P, bf, st, K)
+                      : launch_pass1<__nv_bfloat16, 64>(P, bf, st, K);
+  return P.d == 128 ? launch_pass1<float, 128>(P, bf, st, K) : launch_pass1<float, 64>(P, bf, st, K);
 }
 
 cudaError_t launch_score_simt(const Problem& P, const Buffers& bf, cudaStream_t st,

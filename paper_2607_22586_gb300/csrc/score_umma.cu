@@ -256,6 +256,17 @@ __device__ __forceinline__ void softmax_chunk(float (&v)[32], float alpha, float
   z += zc;
 }
 
+// The same with the reference always at the running max, so no exponent is
+// positive and the largest terms carry no rounding of a large difference: for
+// sums whose ratio is the result (coverage), where the rounding of the
+// selection's sums would not cancel. Costs the max of every chunk.
+__device__ __forceinline__ void softmax_chunk_max(const float (&v)[32], float alpha, float& m, float& z) {
+  const float mn = fmaxf(m, max32(v) * alpha);
+  if (mn == -INFINITY) return;     // every column masked so far
+  z = fmaf(z, fast_exp2(m - mn), exp2_sum32(v, pk2(alpha, alpha), mn));
+  m = mn;
+}
+
 // First chunk of a split: the reference is the chunk's own max (ALU only, so
 // the exponentials are evaluated once); z starts from this chunk's sum.
 __device__ __forceinline__ void softmax_first(const float (&v)[32], float alpha, float& m, float& z) {
@@ -641,7 +652,9 @@ struct PairSmem {
   static constexpr int DYN_BYTES = 1024 + STAT_BYTES + RING_BYTES;
 };
 
-template <int D, bool LISTS>
+// RATIO: the sums feed a ratio (softmax_chunk_max), over at most bf.kept_len
+// keys of each (layer, request, KV head) where given.
+template <int D, bool LISTS, bool RATIO>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     softmax_pair_kernel(const __grid_constant__ CUtensorMap kmap,
                         const __grid_constant__ CUtensorMap pmap, const __grid_constant__ Problem P,
@@ -792,13 +805,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     uint32_t bphase = 0;
     bool ok = true;
     float2* dst = nullptr;
+    int n_keys = 0;                         // keys of the (layer, request, KV head)
     while (ok && walk_next<LISTS>(P, S, wk, nwk, x)) {
       const size_t dst_step = (size_t)kUmmaPartSlots * P.Prows_pad;
-      if (x.fresh)
+      if (x.fresh) {
+        if (RATIO)
+          n_keys = bf.kept_len ? bf.kept_len[((size_t)x.l * P.B + x.b) * P.Hkv + x.h] : x.t_len;
         dst = bf.part + (((size_t)x.l * P.Hkv + x.h) * P.total_splits + P.req[x.b].split_off + x.split) * dst_step +
               (size_t)wg * P.Prows_pad + x.tile * SROWS + (int)rank * PROWS + lrow;
-      else
+      } else {
         dst += dst_step;
+      }
       // (reference max, sum of exp2(x - max)) of this thread's row over its
       // quarter of every tile of the split, restarted per split
       float m_run = -INFINITY, z_run = 0.f;
@@ -810,7 +827,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         fence_after();
         const uint32_t tcol =
             tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * PBK + c_lo);
-        const int nvalid = min(PBK, x.t1 - kt) - c_lo;
+        const int nvalid = min(PBK, (RATIO ? min(x.t1, n_keys) : x.t1) - kt) - c_lo;
         // the accumulator is released as soon as its last columns are in
         // registers, before their exponentials, so the MMAs of the tile after
         // next start half a drain earlier
@@ -825,7 +842,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             if (lane == 0) mbar_arrive_cluster_relaxed(tempty_lead + 8 * buf);
           }
           if (nvalid < PBK / 4) mask_tail(v, c0, nvalid);   // the last tile of a short split
-          if (j == 0 && c0 == 0)
+          if (RATIO)
+            softmax_chunk_max(v, alpha, m_run, z_run);
+          else if (j == 0 && c0 == 0)
             softmax_first(v, alpha, m_run, z_run);
           else
             softmax_chunk(v, alpha, m_run, z_run);
@@ -990,44 +1009,70 @@ int sm_count() {
 static_assert(2 * sizeof(CUtensorMap) + sizeof(Problem) + sizeof(Sched) + sizeof(Buffers) <= 32764,
               "kernel parameters above the 32,764-byte limit");
 
+// Tensor maps of a call: K as 128-key boxes, the packed proxy rows as 16-row
+// boxes.
+template <int D>
+cudaError_t make_maps(const Problem& P, const Buffers& bf, const void* K, CUtensorMap* kmap,
+                      CUtensorMap* pmap) {
+  const uint64_t ls = P.L > 1 ? (uint64_t)P.ls_kv : (uint64_t)P.total_T * P.Hkv * D;
+  if (!make_tmap_bf16_3d(kmap, K, (uint64_t)P.Hkv * D, (uint64_t)P.total_T, (uint64_t)P.L,
+                         (uint64_t)P.Hkv * D * 2, ls * 2, BK))
+    return cudaErrorInvalidValue;
+  if (!make_tmap_bf16_3d(pmap, bf.packed, D, (uint64_t)P.Prows_pad, (uint64_t)P.L * P.B * P.Hkv,
+                         (uint64_t)D * 2, (uint64_t)P.Prows_pad * D * 2, 16))
+    return cudaErrorInvalidValue;
+  return cudaSuccess;
+}
+
+// Softmax pass: workers are CTA pairs (clusters of two), one per two SMs.
+template <int D, bool RATIO>
+cudaError_t launch_softmax_d(const Problem& P, const Buffers& bf, cudaStream_t st,
+                             const CUtensorMap& kmap, const CUtensorMap& pmap, int nsm) {
+  cudaError_t e;
+  for (auto f : {softmax_pair_kernel<D, false, RATIO>, softmax_pair_kernel<D, true, RATIO>})
+    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  PairSmem<D>::DYN_BYTES)) != cudaSuccess) return e;
+  Sched s1 = make_sched(P, 1);
+  if (!s1.units) return cudaSuccess;
+  const int pairs = nsm / 2;
+  if (balance_workers(s1.wl, s1.ntiles, s1.units / s1.ntiles, pairs)) {
+    softmax_pair_kernel<D, true, RATIO><<<2 * pairs, NTHREADS, PairSmem<D>::DYN_BYTES, st>>>(
+        kmap, pmap, P, s1, bf);
+  } else {
+    // whole teams of ntiles pairs
+    const int rows = s1.units / s1.ntiles;
+    const int grid_pairs = std::max(1, std::min(pairs / s1.ntiles, rows)) * s1.ntiles;
+    softmax_pair_kernel<D, false, RATIO><<<2 * grid_pairs, NTHREADS, PairSmem<D>::DYN_BYTES, st>>>(
+        kmap, pmap, P, s1, bf);
+  }
+  return cudaGetLastError();
+}
+
+template <int D>
+cudaError_t launch_softmax_only(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K) {
+  CUtensorMap kmap, pmap;
+  const cudaError_t e = make_maps<D>(P, bf, K, &kmap, &pmap);
+  if (e != cudaSuccess) return e;
+  const int nsm = sm_count();
+  if (nsm <= 0) return cudaErrorInvalidDevice;
+  return launch_softmax_d<D, true>(P, bf, st, kmap, pmap, nsm);
+}
+
 template <int D>
 cudaError_t launch_d(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K,
                      cudaEvent_t* ev) {
   using SM = Smem<D>;
   CUtensorMap kmap, pmap;
-  const uint64_t ls = P.L > 1 ? (uint64_t)P.ls_kv : (uint64_t)P.total_T * P.Hkv * D;
-  if (!make_tmap_bf16_3d(&kmap, K, (uint64_t)P.Hkv * D, (uint64_t)P.total_T, (uint64_t)P.L,
-                   (uint64_t)P.Hkv * D * 2, ls * 2, BK))
-    return cudaErrorInvalidValue;
-  if (!make_tmap_bf16_3d(&pmap, bf.packed, D, (uint64_t)P.Prows_pad, (uint64_t)P.L * P.B * P.Hkv,
-                   (uint64_t)D * 2, (uint64_t)P.Prows_pad * D * 2, 16))
-    return cudaErrorInvalidValue;
+  cudaError_t e = make_maps<D>(P, bf, K, &kmap, &pmap);
+  if (e != cudaSuccess) return e;
   const int nsm = sm_count();
   if (nsm <= 0) return cudaErrorInvalidDevice;
-  cudaError_t e;
-  for (auto f : {softmax_pair_kernel<D, false>, softmax_pair_kernel<D, true>})
-    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  PairSmem<D>::DYN_BYTES)) != cudaSuccess) return e;
   for (auto f : {mass_umma_kernel<D, false>, mass_umma_kernel<D, true>})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   SM::DYN_BYTES)) != cudaSuccess) return e;
-  Sched s1 = make_sched(P, 1), s2 = make_sched(P, 2);
+  Sched s2 = make_sched(P, 2);
   if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
-  if (s1.units) {
-    // softmax pass: workers are CTA pairs (clusters of two), one per two SMs
-    const int pairs = nsm / 2;
-    if (balance_workers(s1.wl, s1.ntiles, s1.units / s1.ntiles, pairs)) {
-      softmax_pair_kernel<D, true><<<2 * pairs, NTHREADS, PairSmem<D>::DYN_BYTES, st>>>(
-          kmap, pmap, P, s1, bf);
-    } else {
-      // whole teams of ntiles pairs
-      const int rows = s1.units / s1.ntiles;
-      const int grid_pairs = std::max(1, std::min(pairs / s1.ntiles, rows)) * s1.ntiles;
-      softmax_pair_kernel<D, false><<<2 * grid_pairs, NTHREADS, PairSmem<D>::DYN_BYTES, st>>>(
-          kmap, pmap, P, s1, bf);
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  }
+  if ((e = launch_softmax_d<D, false>(P, bf, st, kmap, pmap, nsm)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   if ((e = launch_merge(P, bf, st)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
@@ -1076,15 +1121,19 @@ bool make_tmap_bf16_3d(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d
 
 bool tmap_encoder_available() { return encode_fn() != nullptr; }
 
-bool umma_supported(const Problem& P) {
-  if (P.dtype != MMSHIFT_BF16 || (P.d != 64 && P.d != 128)) return false;
-  if (P.RG > SROWS || P.anchor_rows > SROWS || P.Prows_pad % SROWS) return false;
+bool umma_softmax_supported(const Problem& P) {
+  if (P.dtype != MMSHIFT_BF16 || (P.d != 64 && P.d != 128) || P.Prows_pad % SROWS) return false;
   if (P.L > 1 && (P.ls_kv % 8)) return false;   // TMA strides: multiples of 16 bytes
   int dev = 0, major = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess)
     return false;
   return major == 10 && tmap_encoder_available();
+}
+
+// The mass pass also needs whole groups within a stationary block.
+bool umma_supported(const Problem& P) {
+  return P.RG <= SROWS && P.anchor_rows <= SROWS && umma_softmax_supported(P);
 }
 
 int umma_launches(const Problem& P) { return P.anchor_split ? 5 : 3; }
@@ -1098,6 +1147,12 @@ cudaError_t launch_anchor_split(const Problem& P, const Buffers& bf, cudaStream_
   if (e != cudaSuccess) return e;
   anchor_final_kernel<<<dim3(P.total_splits, P.Hkv, P.L), ANT, 0, st>>>(P, bf);
   return cudaGetLastError();
+}
+
+cudaError_t launch_softmax_umma(const Problem& P, const Buffers& bf, cudaStream_t st,
+                                const void* K) {
+  if (reinterpret_cast<uintptr_t>(K) & 15) return cudaErrorMisalignedAddress;
+  return P.d == 128 ? launch_softmax_only<128>(P, bf, st, K) : launch_softmax_only<64>(P, bf, st, K);
 }
 
 cudaError_t launch_score_umma(const Problem& P, const Buffers& bf, cudaStream_t st,

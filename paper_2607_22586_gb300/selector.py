@@ -105,7 +105,12 @@ class KVSelector:
         self._check(K, qwin, dec_q)
         n_dec = dec_q.shape[3]
         n = L.mmshift_coverage_workspace_size(self.shape, n_dec)
-        ws = torch.zeros(n, dtype=torch.uint8, device=self.device)
+        # only the status word, in the first 256 bytes, has to start at zero
+        if n <= 1 << 23:
+            ws = torch.zeros(n, dtype=torch.uint8, device=self.device)
+        else:
+            ws = torch.empty(n, dtype=torch.uint8, device=self.device)
+            ws[:256].zero_()
         out = torch.empty((self.n_layers, len(self.budgets), self.n_kv_heads, n_dec),
                           dtype=torch.float32, device=self.device)
         L.check(L.mmshift_coverage(self.shape, K, qwin, dec_q, n_dec, softmax_scale,
