@@ -21,6 +21,7 @@
 //    (ties: lower t) and an ordered compaction with warp ballots that writes
 //    the kept indices ascending with T-1 last.
 #include "common.cuh"
+#include "umma.cuh"
 
 namespace mmshift {
 namespace {
@@ -61,6 +62,8 @@ struct SelShared {
   unsigned int ncand;
   unsigned int rend;
   int aux;
+  unsigned long long gspec, target, lb;   // cover_kernel's bounds
+  bool again;
 };
 
 // Key sources, chosen at compile time: keys staged in shared memory, or
@@ -458,14 +461,43 @@ __device__ void total_and_max(const float* m, int n, int shift, uint32_t kspec, 
   const uint32_t wmin = ordered_key(__int_as_float((126 - shift) << 23)) + 1u;
   unsigned long long tot = 0;
   uint32_t km = 0;
+  auto weight = [&](uint32_t k) { return k >= wmin ? fx_weight(k, shift) : 0ull; };
   auto append = [&](uint32_t k, int i) {
     const unsigned o = atomicAdd(&S.ncand, 1u);
     if (o < (unsigned)cap) { cand[o] = k; cidx[o] = (uint32_t)i; }
   };
+  // Weights of x0, x1 in [0, 32) in 2^-40 units by float32 adds, instead of
+  // fx_weight's 30 integer instructions each: x + 96 rounds x to a multiple a
+  // of 2^-17, x - a is exact and at most 2^-18, and (x - a) 2^40 + 1.5 2^23 (one
+  // FMA) holds its nearest integer, halves to even, in its low bits. x 2^40
+  // rounds the same way, since a 2^40 is an even integer. th sums a in 2^-17
+  // units, tl the rest: th 2^23 + tl in all, exactly fx_weight's.
+  // With the warp-wide key_of_weight and one warp's scalar work, coverage vote of
+  // the 28-layer 32K stack 156 -> 121 us, few proxies 26.5 -> 18.3 us (issue-bound
+  // on what is left of the pass: clamps, maxima, the ring).
+  constexpr uint32_t kFast = 0xC2000000u;      // key of 32
+  constexpr int kCarry = 64;                   // quads between carries: |th|, |tl| <= 2^30
+  uint32_t th = 0, tl = 0, nq = 0;             // sums of the bit patterns, mod 2^32
+  auto carry = [&] {
+    const int32_t a = (int32_t)(th - 4u * nq * 0x42C00000u);   // less 96 per key
+    const int32_t f = (int32_t)(tl - 4u * nq * 0x4B400000u);   // less 1.5 2^23 per key
+    tot += ((unsigned long long)(long long)a << 23) + (unsigned long long)(long long)f;
+    th = tl = nq = 0;
+  };
+  auto add2 = [&](float x0, float x1) {
+    const uint64_t x = umma::pk2(x0, x1);
+    const uint64_t c = umma::pk2(96.f, 96.f), nc = umma::pk2(-96.f, -96.f);
+    const uint64_t t = umma::fadd2(x, c);
+    const uint64_t na = umma::ffma2(umma::fadd2(t, nc), umma::pk2(-1.f, -1.f), x);   // x - a
+    const uint64_t f = umma::ffma2(na, umma::pk2(1099511627776.f, 1099511627776.f),
+                                   umma::pk2(12582912.f, 12582912.f));
+    th += (uint32_t)t + (uint32_t)(t >> 32);
+    tl += (uint32_t)f + (uint32_t)(f >> 32);
+  };
   auto add1 = [&](float x, int i) {
     const uint32_t k = nonneg_key(x);
     km = max(km, k);
-    if (k >= wmin) tot += fx_weight(k, shift);
+    tot += weight(k);
     if (k >= kspec) append(k, i);
   };
   const int head = min(n, (int)(((16u - (uint32_t)(reinterpret_cast<uintptr_t>(m) & 15)) & 15u) >> 2));
@@ -484,20 +516,23 @@ __device__ void total_and_max(const float* m, int n, int shift, uint32_t kspec, 
     const int i4 = c * NTH + tid;
     if (i4 < n4) {
       const float4 f = ring[slot * NTH + tid];
-      const uint32_t k0 = nonneg_key(f.x), k1 = nonneg_key(f.y), k2 = nonneg_key(f.z),
-                     k3 = nonneg_key(f.w);
-      km = max(max(km, max(k0, k1)), max(k2, k3));
-      const unsigned long long w0 = k0 >= wmin ? fx_weight(k0, shift) : 0ull;
-      const unsigned long long w1 = k1 >= wmin ? fx_weight(k1, shift) : 0ull;
-      const unsigned long long w2 = k2 >= wmin ? fx_weight(k2, shift) : 0ull;
-      const unsigned long long w3 = k3 >= wmin ? fx_weight(k3, shift) : 0ull;
-      tot += (w0 + w1) + (w2 + w3);
-      if (max(max(k0, k1), max(k2, k3)) >= kspec) {   // rare
+      const float x0 = fmaxf(f.x, 0.f), x1 = fmaxf(f.y, 0.f), x2 = fmaxf(f.z, 0.f), x3 = fmaxf(f.w, 0.f);
+      const uint32_t kq = ordered_key(fmaxf(fmaxf(x0, x1), fmaxf(x2, x3)));
+      km = max(km, kq);
+      if (shift == 40 && kq < kFast) {
+        add2(x0, x1);
+        add2(x2, x3);
+        if (++nq == kCarry) carry();
+      } else {
+        tot += (weight(ordered_key(x0)) + weight(ordered_key(x1))) +
+               (weight(ordered_key(x2)) + weight(ordered_key(x3)));
+      }
+      if (kq >= kspec) {   // rare
         const int i0 = head + 4 * i4;
-        if (k0 >= kspec) append(k0, i0);
-        if (k1 >= kspec) append(k1, i0 + 1);
-        if (k2 >= kspec) append(k2, i0 + 2);
-        if (k3 >= kspec) append(k3, i0 + 3);
+        if (ordered_key(x0) >= kspec) append(ordered_key(x0), i0);
+        if (ordered_key(x1) >= kspec) append(ordered_key(x1), i0 + 1);
+        if (ordered_key(x2) >= kspec) append(ordered_key(x2), i0 + 2);
+        if (ordered_key(x3) >= kspec) append(ordered_key(x3), i0 + 3);
       }
     }
     // the quad this thread just read is in registers: its slot takes the
@@ -507,6 +542,7 @@ __device__ void total_and_max(const float* m, int n, int shift, uint32_t kspec, 
     cp_async_commit();
     if (++slot == kRingStages) slot = 0;
   }
+  carry();
   cp_async_wait<0>();
   for (int i = head + (n4 << 2) + tid; i < n; i += NTH) add1(__ldg(m + i), i);
   for (int off = 16; off; off >>= 1) {
@@ -522,12 +558,21 @@ __device__ void total_and_max(const float* m, int n, int shift, uint32_t kspec, 
 }
 
 // Smallest key (of a non-negative float) whose weight in 2^-shift units is
-// at least wt >= 1 (weights do not decrease with the key).
+// at least wt >= 1 (weights do not decrease with the key), by a whole warp: 32
+// probes a round, so seven rounds instead of 31 steps of one thread.
 __device__ __forceinline__ uint32_t key_of_weight(unsigned long long wt, int shift) {
+  const uint32_t lane = threadIdx.x & 31;
   uint32_t lo = 0x80000001u, hi = 0xFF7FFFFFu;   // the largest finite float weighs >= 2^63
   while (lo < hi) {
-    const uint32_t mid = lo + ((hi - lo) >> 1);
-    if (fx_weight(mid, shift) >= wt) hi = mid; else lo = mid + 1u;
+    const uint32_t step = (hi - lo) / 32u + 1u;
+    const uint32_t off = lane * step;            // at most 31 * 2^26
+    const uint32_t probe = off < hi - lo ? lo + off : hi;
+    const unsigned ge = __ballot_sync(0xffffffffu, fx_weight(probe, shift) >= wt);
+    const int f = ge ? __ffs(ge) - 1 : 32;       // first probe that weighs enough
+    const uint32_t at = __shfl_sync(0xffffffffu, probe, f & 31);
+    const uint32_t below = __shfl_sync(0xffffffffu, probe, (f - 1) & 31);
+    if (f < 32) hi = at;
+    if (f > 0) lo = min(below + 1u, hi);
   }
   return lo;
 }
@@ -698,18 +743,24 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) cover_kernel(Problem P, Buffe
   // total implies are collected in the same pass as the total; the
   // collection stands if its bound is at most lb, else a second pass
   // collects the keys of weight >= lb.
+  // One warp does the scalar work in float64 and 64-bit integers (a warp's
+  // float64 instruction holds the SM's unit for 16 clocks).
   int shift = 40;
-  unsigned long long gspec = 0;
-  if (P.cover_hint > 0.f) {
-    const double g = ((1.0 - (double)P.tau) * 0.5 * (double)P.cover_hint * 1099511627776.0 - 1.0) /
-                     (double)n;                       // 2^40 units
-    gspec = g >= 1.0 ? (unsigned long long)g : 0ull;
-  }
-  if (tid == 0) {
-    S.prefix = gspec ? key_of_weight(gspec, shift) : 0xFFFFFFFFu;
-    S.ncand = 0;
-    S.cum_w = 0;
-    S.cum_n = 0;
+  if (tid < 32) {
+    unsigned long long gspec = 0;
+    if (P.cover_hint > 0.f) {
+      const double g = ((1.0 - (double)P.tau) * 0.5 * (double)P.cover_hint * 1099511627776.0 - 1.0) /
+                       (double)n;                       // 2^40 units
+      gspec = g >= 1.0 ? (unsigned long long)g : 0ull;
+    }
+    const uint32_t k = gspec ? key_of_weight(gspec, shift) : 0xFFFFFFFFu;
+    if (tid == 0) {
+      S.gspec = gspec;
+      S.prefix = k;
+      S.ncand = 0;
+      S.cum_w = 0;
+      S.cum_n = 0;
+    }
   }
   for (int i = tid; i < (n + 31) / 32; i += NTH) bits[i] = 0u;
   __syncthreads();
@@ -718,6 +769,7 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) cover_kernel(Problem P, Buffe
   total_and_max<NTH>(m, n, shift, S.prefix, cand, cidx, kCoverCand,
                      reinterpret_cast<float4*>(hist), S, total, kmax);
   int nc = (int)S.ncand;
+  unsigned long long gspec = S.gspec;
   {
     // the 2^-shift unit is lowered where n * max * 2^shift could overflow 64 bits
     int e = 0;
@@ -731,19 +783,27 @@ __global__ void __launch_bounds__(NTH, 1024 / NTH) cover_kernel(Problem P, Buffe
                          reinterpret_cast<float4*>(hist), S, total, kmax);
     }
   }
-  const unsigned long long tt = (unsigned long long)ceil((double)P.tau * (double)total);
-  unsigned long long target_w = tt > total ? total : tt;
-  const unsigned long long lb = (total - target_w + 1) / (unsigned long long)n;
-  if (lb > 0) {
-    if (!(gspec > 0 && gspec <= lb && nc <= kCoverCand)) {
-      __syncthreads();   // every thread has read S.ncand
-      if (tid == 0) {
-        S.prefix = key_of_weight(lb, shift);
-        S.ncand = 0;
-      }
-      __syncthreads();
-      nc = compact_above<NTH>(m, n, S.prefix, cand, cidx, kCoverCand, S);
+  if (tid < 32) {
+    const unsigned long long tt = (unsigned long long)ceil((double)P.tau * (double)total);
+    const unsigned long long target = tt > total ? total : tt;
+    const unsigned long long lb = (total - target + 1) / (unsigned long long)n;
+    const bool again = lb > 0 && !(gspec > 0 && gspec <= lb && nc <= kCoverCand);
+    // the other warps' nc is not used when S.ncand restarts: they take
+    // compact_above's count
+    const uint32_t k = again ? key_of_weight(lb, shift) : 0u;
+    if (tid == 0) {
+      S.target = target;
+      S.lb = lb;
+      S.again = again;
+      if (again) { S.prefix = k; S.ncand = 0; }
     }
+  }
+  __syncthreads();
+  unsigned long long target_w = S.target;
+  const unsigned long long lb = S.lb;
+  if (lb > 0) {
+    if (S.again)
+      nc = compact_above<NTH>(m, n, S.prefix, cand, cidx, kCoverCand, S);
     if (nc > 0 && nc <= kCoverCand) {
       cover_among<NTH>(cand, cidx, nc, 0, 0x80000000u, target_w, shift, P.tau, S, hist, bits);
       return;
