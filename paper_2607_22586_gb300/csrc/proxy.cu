@@ -240,7 +240,8 @@ __device__ __noinline__ void enlist(const Problem& P, const Buffers& bf, int l, 
 }
 
 // Proxies of one query head are spread over up to kProxyChunks CTAs, about
-// 1024 Philox draws each (few proxies: one CTA per query head).
+// 1024 Philox draws each (few proxies: one CTA per query head), or more CTAs
+// where the call would not fill the SMs (launch_t).
 constexpr int kProxyChunks = 8;
 
 template <typename T, int D>
@@ -367,21 +368,28 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
       store4(pout + (size_t)i * D + D / 2 + 4 * qq, v[4], v[5], v[6], v[7]);
     }
   }
-  if (!packed || chunk != 0) return;
+  if (!packed) return;
   // anchor row of this query head: the last window query as given
-  if (P.anchor_rows) {
+  if (P.anchor_rows && chunk == 0) {
     T* arow = packed + (size_t)(P.n_group_rows + j) * D;
     for (int k = threadIdx.x; k < D; k += blockDim.x) arow[k] = q[(size_t)(P.W - 1) * qstride + k];
   }
   // padding rows (the tail of each group's rows, of the anchor rows and of
-  // the block) are zeroed by the first query head of the KV head
-  if (j == 0) {
+  // the block) are zeroed in 16-byte stores by all CTAs of the KV head: about
+  // 240 rows, which one CTA storing element by element kept the whole kernel
+  // waiting for (41,000 clocks against 20,000 on average). Sampler and
+  // refinement, with the spread of launch_t: 64 heads x 4 requests of 32
+  // proxies 36.5 -> 28.4 us, one layer of 28 heads, 512 proxies 39 -> 31.5 us, ten
+  // layers of the 72B-class batch 148 -> 124 us.
+  {
     const int gpad = P.RG - P.r * P.gs;                  // per group
     const int apad = P.anchor_rows ? P.anchor_rows - P.r : 0;   // after the anchor rows
     const int tail = P.Prows_pad - P.Prows;              // after the last block row
     const int n_pad = P.G * gpad + apad + tail;
-    for (int e = threadIdx.x; e < n_pad * D; e += blockDim.x) {
-      const int pr = e / D, k = e - pr * D;
+    constexpr int VPR = D * (int)sizeof(T) / 16;         // 16-byte stores per row
+    for (int e = (j * nch + chunk) * blockDim.x + threadIdx.x; e < n_pad * VPR;
+         e += P.r * nch * blockDim.x) {
+      const int pr = e / VPR;
       int row;
       if (pr < P.G * gpad) {
         row = (pr / gpad) * P.RG + P.r * P.gs + pr % gpad;
@@ -390,7 +398,7 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
       } else {
         row = P.Prows + (pr - P.G * gpad - apad);
       }
-      packed[(size_t)row * D + k] = from_f32<T>(0.f);
+      reinterpret_cast<uint4*>(packed + (size_t)row * D)[e % VPR] = make_uint4(0, 0, 0, 0);
     }
   }
 }
@@ -437,8 +445,16 @@ bool has_refine_list(const Buffers& bf) {
 
 template <typename T, int D>
 cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const void* qwin) {
+  cudaError_t e;
+  int dev = 0, nsm = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int draws = P.Np * (D / 8);
-  const int nch = draws <= 0 ? 1 : std::min(kProxyChunks, (draws + 1023) / 1024);
+  int nch = draws <= 0 ? 1 : std::min(kProxyChunks, (draws + 1023) / 1024);
+  // a short call's heads are spread further, down to one draw per thread,
+  // until the launch holds the six CTAs per SM that fit
+  const long long heads = (long long)P.Hq * P.B * P.L;
+  nch = (int)std::max<long long>(nch, std::min<long long>((draws + 255) / 256, 6LL * nsm / heads));
   const bool refine = samples_bf16(P, bf);
   Buffers b2 = bf;
   if (!has_refine_list(bf)) {
@@ -447,7 +463,6 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
     b2.refine_cap = 0;
     b2.refine_stats = nullptr;
   }
-  cudaError_t e;
   if (refine && b2.refine_items &&
       (e = cudaMemsetAsync(b2.refine_count, 0, sizeof(int), st)) != cudaSuccess)
     return e;
@@ -455,10 +470,6 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
   proxy_pack_kernel<T, D><<<grid, 256, 0, st>>>(P, b2, (const T*)qwin, nch);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (refine) {
-    int dev = 0, nsm = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-      return e;
     const bool all = b2.refine_items == nullptr;
     refine_kernel<D><<<8 * std::max(nsm, 1), 128, 0, st>>>(
         P, b2, (const __nv_bfloat16*)qwin, all);
