@@ -320,8 +320,9 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
   constexpr int NQ8 = D / 8;  // threads per proxy: dims [4qq, 4qq+4) and [D/2+4qq, +4)
   const int per = (P.Np + nch - 1) / nch;
   const int i0 = chunk * per, i1 = min(P.Np, i0 + per);
-  // independent iterations unrolled so several Philox chains are in flight
-#pragma unroll 4
+  // two iterations at once, so two Philox chains are in flight (four: 240 us
+  // against 233 on the 8K stack)
+#pragma unroll 2
   for (int e = i0 * NQ8 + threadIdx.x; e < i1 * NQ8; e += blockDim.x) {
     const int i = e / NQ8, qq = e - i * NQ8;
     float v[8];
