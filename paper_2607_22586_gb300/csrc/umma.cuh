@@ -258,6 +258,13 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t caddr) {
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t caddr) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(caddr) : "memory");
 }
+// A role that gave up tells its CTA and the pair's other one (the flag at the
+// same offset there), so that no role of either waits out its limit.
+__device__ __forceinline__ void abort_pair(int* flag, uint32_t other) {
+  *reinterpret_cast<volatile int*>(flag) = 1;
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(smem_u32(flag), other)), "r"(1)
+               : "memory");
+}
 // TMA tile load into this CTA's shared memory whose completion is counted on
 // an mbarrier of either CTA of the pair (cluster address).
 __device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* map, uint32_t bar_caddr,
