@@ -216,12 +216,21 @@ int choose_umma(const Problem& P, const void* K) {
   return (umma_supported(P) && (reinterpret_cast<uintptr_t>(K) & 15) == 0) ? 1 : 0;
 }
 
+// A call is short when a scoring pass has at most this many units (key splits x
+// 256-row blocks x heads x layers; 76 CTA pairs take them): its kernels are then
+// launched as programmatic dependents. One layer of 4096 keys (240 units) 108 ->
+// 96.5 us, steps 2-4 on 4,500 keys 53 -> 44 us, two layers of 8192 keys (960 units)
+// 185 -> 179.5 us; the 28-layer stacks (13,440 and 53,760 units) lose 1-2%.
+constexpr long long kShortCall = 1024;
+
 // Scoring path of a call: tensor or CUDA cores, and the softmax partials
-// and anchor handling that go with it.
+// and anchor handling that go with it; whether its kernels overlap.
 void set_score_path(Problem& P, const void* K) {
   P.use_umma = choose_umma(P, K);
   P.part_slots = P.use_umma ? kUmmaPartSlots : 1;
   P.anchor_split = P.use_umma && anchor_spills(P) ? 1 : 0;
+  const long long units = (long long)P.L * P.Hkv * P.total_splits * (P.Prows_pad / kRowTile);
+  P.overlap = units <= kShortCall;
 }
 
 // Kernels one mmshift_select call enqueues (reported through mmshift_debug).

@@ -62,6 +62,9 @@ struct Problem {
   // each row's softmax sums to 1) when the coverage vote reads masses this
   // library computed, else 0 (set per call); only a hint, checked in use
   float cover_hint;
+  // a short call: its kernels are launched as programmatic dependents of one
+  // another (set per call, see launch_kernel)
+  int32_t overlap;
   int32_t test_stuck_wait; // test only: see mmshift_debug.test_stuck_wait
   ReqInfo req[MMSHIFT_MAX_BATCH];
 };
@@ -178,6 +181,48 @@ __device__ __forceinline__ void merge_ms(float& m, float& z, float m2, float z2)
 
 __device__ __forceinline__ void set_status(int* status, int bit) {
   if (status) atomicOr(status, bit);
+}
+
+// Start of every kernel that may be launched as a programmatic dependent: the
+// next kernel of the call may take its place on the SMs, and everything the
+// kernels before this one wrote is visible afterwards. Without the launch
+// attribute both are no-ops.
+__device__ __forceinline__ void dependent_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Launches a kernel, with cluster > 1 in clusters along x. `overlap`: as a
+// programmatic dependent of the kernel before it in the stream, whose
+// launch latency then overlaps that kernel (both start with dependent_start,
+// so a kernel still begins its work after the one before it has finished).
+// Short calls use it: about 1 us per kernel of a ten-kernel call. Long ones do
+// not: waiting CTAs take places and issue slots from kernels that fill the SMs.
+template <class... KP, class... A>
+cudaError_t launch_kernel(void (*k)(KP...), dim3 grid, unsigned block, size_t smem, cudaStream_t st,
+                          bool overlap, int cluster, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  unsigned n = 0;
+  if (cluster > 0) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = (unsigned)cluster;
+    at[n].val.clusterDim.y = 1;
+    at[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (overlap) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, k, static_cast<KP>(args)...);
 }
 
 // Host-side launchers (one translation unit each).

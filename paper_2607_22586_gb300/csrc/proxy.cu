@@ -207,6 +207,7 @@ constexpr int kProxyChunks = 8;
 template <typename T, int D>
 __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers bf, const T* qwin,
                                                          int nch) {
+  dependent_start();
   const int hq = blockIdx.x / nch, chunk = blockIdx.x % nch;
   const int b = blockIdx.y, l = blockIdx.z;
   const int h = hq / P.r, j = hq - h * P.r;
@@ -378,6 +379,7 @@ template <int D>
 __global__ void __launch_bounds__(224) refine_kernel(const __grid_constant__ Problem P,
                                                      const __grid_constant__ Buffers bf,
                                                      const __nv_bfloat16* qwin, bool all) {
+  dependent_start();
   __shared__ double mu[2][32], sig[2][32], rad[2][32], trig[2][32], rot[2][32];
   constexpr int half = D / 2;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -495,9 +497,8 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (refine) {
     const bool all = b2.refine_items == nullptr;
-    refine_kernel<D><<<8 * std::max(nsm, 1), P.rope_theta > 0.f ? 224 : 96, 0, st>>>(
-        P, b2, (const __nv_bfloat16*)qwin, all);
-    e = cudaGetLastError();
+    e = launch_kernel(refine_kernel<D>, dim3(8 * std::max(nsm, 1)), P.rope_theta > 0.f ? 224 : 96, 0,
+                      st, P.overlap, 0, P, b2, (const __nv_bfloat16*)qwin, all);
   }
   return e;
 }

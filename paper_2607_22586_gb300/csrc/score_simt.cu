@@ -158,6 +158,7 @@ __device__ __forceinline__ void cluster_barrier() {
 template <typename T, int D>
 __global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Problem P, Buffers bf,
                                                   const T* K, int nrank, bool vec) {
+  dependent_start();
   extern __shared__ float sm[];
   float* As = sm;                    // [D][64] proxy rows
   float* Bs = As + TR * D;           // [2][KC][128] keys, a piece and the next one
@@ -278,7 +279,8 @@ __global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Pro
 // shuffles; for a given SUB the order is fixed, and SUB depends only on the
 // call's shape.
 template <int kMergeSub>
-__global__ void merge_kernel(Problem P, Buffers bf) {
+__global__ void merge_kernel(const __grid_constant__ Problem P, const __grid_constant__ Buffers bf) {
+  dependent_start();
   const int q = threadIdx.x % kMergeSub;
   const int p = blockIdx.x * (blockDim.x / kMergeSub) + threadIdx.x / kMergeSub;
   const int bh = blockIdx.y, l = blockIdx.z;
@@ -319,6 +321,7 @@ __global__ void merge_kernel(Problem P, Buffers bf) {
 template <typename T, int D>
 __global__ void __launch_bounds__(TNT, 2) pass2_simt(const __grid_constant__ Problem P, Buffers bf,
                                                   const T* K, int gper, bool vec) {
+  dependent_start();
   extern __shared__ float sm[];
   float* Bs = sm;                    // [D][128] keys (stationary)
   float* As = Bs + TK * D;           // [2][KC][64] proxy rows, a piece and the next one
@@ -455,19 +458,8 @@ cudaError_t launch_pass1(const Problem& P, const Buffers& bf, cudaStream_t st, c
   const size_t sm1 = (size_t)(TR * D + 2 * KC * TK) * sizeof(float) + (size_t)runs * TR * sizeof(float2);
   if ((e = cudaFuncSetAttribute(pass1_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sm1)) != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(P.Hkv * P.total_splits * n_rt * nrank), P.L);
-  cfg.blockDim = dim3(TNT);
-  cfg.dynamicSmemBytes = sm1;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = nrank;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, pass1_simt<T, D>, P, bf, (const T*)K, nrank, vec);
+  return launch_kernel(pass1_simt<T, D>, dim3((unsigned)(P.Hkv * P.total_splits * n_rt * nrank), P.L), TNT,
+                       sm1, st, P.overlap, nrank, P, bf, (const T*)K, nrank, vec);
 }
 
 template <typename T, int D>
@@ -493,9 +485,8 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
   const size_t sm2 = (size_t)(TK * D + 2 * KC * TR + 4 * TK) * sizeof(float);
   if ((e = cudaFuncSetAttribute(pass2_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sm2)) != cudaSuccess) return e;
-  pass2_simt<T, D><<<dim3((unsigned)(tiles * P.Hkv * ngr), P.L), TNT, sm2, st>>>(P, bf, (const T*)K,
-                                                                              gper, vec);
-  return cudaGetLastError();
+  return launch_kernel(pass2_simt<T, D>, dim3((unsigned)(tiles * P.Hkv * ngr), P.L), TNT, sm2, st,
+                       P.overlap, 0, P, bf, (const T*)K, gper, vec);
 }
 
 }  // namespace
@@ -507,13 +498,12 @@ cudaError_t launch_merge(const Problem& P, const Buffers& bf, cudaStream_t st) {
   if (max_ns >= 128) {
     constexpr int threads = 256, rows_per_block = threads / 4;
     dim3 grid((rows + rows_per_block - 1) / rows_per_block, P.B * P.Hkv, P.L);
-    merge_kernel<4><<<grid, threads, 0, st>>>(P, bf);
+    return launch_kernel(merge_kernel<4>, grid, threads, 0, st, P.overlap, 0, P, bf);
   } else {
     constexpr int threads = 128;
     dim3 grid((rows + threads - 1) / threads, P.B * P.Hkv, P.L);
-    merge_kernel<1><<<grid, threads, 0, st>>>(P, bf);
+    return launch_kernel(merge_kernel<1>, grid, threads, 0, st, P.overlap, 0, P, bf);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_softmax_simt(const Problem& P, const Buffers& bf, cudaStream_t st,

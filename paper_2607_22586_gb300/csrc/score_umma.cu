@@ -441,6 +441,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   fence_after();
   const uint32_t tmem = tbase;
+  dependent_start();   // barriers and tensor memory are ready by now
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
@@ -706,6 +707,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
   cluster_sync();   // both CTAs' barriers exist before any remote arrival
   fence_after();
   const uint32_t tmem = tbase;
+  dependent_start();   // barriers and tensor memory are ready by now
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer (both CTAs)
@@ -882,7 +884,8 @@ __device__ __forceinline__ int split_request(const Problem& P, int s) {
 
 // warp j: anchor row j over the split's keys, 32 keys per round
 __global__ void __launch_bounds__(ANT) anchor_part_kernel(const __grid_constant__ Problem P,
-                                                          Buffers bf) {
+                                                          const __grid_constant__ Buffers bf) {
+  dependent_start();
   const int s = blockIdx.x, h = blockIdx.y, l = blockIdx.z;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (w >= P.r) return;
@@ -919,7 +922,8 @@ __global__ void __launch_bounds__(ANT) anchor_part_kernel(const __grid_constant_
 }
 
 __global__ void __launch_bounds__(ANT) anchor_final_kernel(const __grid_constant__ Problem P,
-                                                           Buffers bf) {
+                                                           const __grid_constant__ Buffers bf) {
+  dependent_start();
   const int s = blockIdx.x, h = blockIdx.y, l = blockIdx.z;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const ReqInfo R = P.req[split_request(P, s)];
@@ -1036,16 +1040,15 @@ cudaError_t launch_softmax_d(const Problem& P, const Buffers& bf, cudaStream_t s
   if (!s1.units) return cudaSuccess;
   const int pairs = nsm / 2;
   if (balance_workers(s1.wl, s1.ntiles, s1.units / s1.ntiles, pairs)) {
-    softmax_pair_kernel<D, true, RATIO><<<2 * pairs, NTHREADS, PairSmem<D>::DYN_BYTES, st>>>(
-        kmap, pmap, P, s1, bf);
+    return launch_kernel(softmax_pair_kernel<D, true, RATIO>, dim3(2 * pairs), NTHREADS,
+                         PairSmem<D>::DYN_BYTES, st, P.overlap, 0, kmap, pmap, P, s1, bf);
   } else {
     // whole teams of ntiles pairs
     const int rows = s1.units / s1.ntiles;
     const int grid_pairs = std::max(1, std::min(pairs / s1.ntiles, rows)) * s1.ntiles;
-    softmax_pair_kernel<D, false, RATIO><<<2 * grid_pairs, NTHREADS, PairSmem<D>::DYN_BYTES, st>>>(
-        kmap, pmap, P, s1, bf);
+    return launch_kernel(softmax_pair_kernel<D, false, RATIO>, dim3(2 * grid_pairs), NTHREADS,
+                         PairSmem<D>::DYN_BYTES, st, P.overlap, 0, kmap, pmap, P, s1, bf);
   }
-  return cudaGetLastError();
 }
 
 template <int D>
@@ -1079,13 +1082,15 @@ cudaError_t launch_d(const Problem& P, const Buffers& bf, cudaStream_t st, const
   if (s2.units) {
     // mass pass: workers are CTAs, one per SM
     if (balance_workers(s2.wl, s2.ntiles, s2.units / s2.ntiles, nsm)) {
-      mass_umma_kernel<D, true><<<nsm, NTHREADS, SM::DYN_BYTES, st>>>(kmap, pmap, P, s2, bf);
+      e = launch_kernel(mass_umma_kernel<D, true>, dim3(nsm), NTHREADS, SM::DYN_BYTES, st, P.overlap, 0,
+                        kmap, pmap, P, s2, bf);
     } else {
       const int rows = s2.units / s2.ntiles;
       const int grid = std::max(1, std::min(nsm / s2.ntiles, rows)) * s2.ntiles;
-      mass_umma_kernel<D, false><<<grid, NTHREADS, SM::DYN_BYTES, st>>>(kmap, pmap, P, s2, bf);
+      e = launch_kernel(mass_umma_kernel<D, false>, dim3(grid), NTHREADS, SM::DYN_BYTES, st, P.overlap, 0,
+                        kmap, pmap, P, s2, bf);
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -1142,11 +1147,10 @@ int umma_launches(const Problem& P) { return P.anchor_split ? 5 : 3; }
 // stage, so that the mass pass is timed alone).
 cudaError_t launch_anchor_split(const Problem& P, const Buffers& bf, cudaStream_t st) {
   if (!P.anchor_split || !P.total_T) return cudaSuccess;
-  anchor_part_kernel<<<dim3(P.total_splits, P.Hkv, P.L), ANT, 0, st>>>(P, bf);
-  cudaError_t e = cudaGetLastError();
+  const dim3 grid(P.total_splits, P.Hkv, P.L);
+  const cudaError_t e = launch_kernel(anchor_part_kernel, grid, ANT, 0, st, P.overlap, 0, P, bf);
   if (e != cudaSuccess) return e;
-  anchor_final_kernel<<<dim3(P.total_splits, P.Hkv, P.L), ANT, 0, st>>>(P, bf);
-  return cudaGetLastError();
+  return launch_kernel(anchor_final_kernel, grid, ANT, 0, st, P.overlap, 0, P, bf);
 }
 
 cudaError_t launch_softmax_umma(const Problem& P, const Buffers& bf, cudaStream_t st,

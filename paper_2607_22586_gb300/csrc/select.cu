@@ -717,7 +717,8 @@ __device__ void cover_among(const uint32_t* cand, const uint32_t* cidx, int nc, 
 }
 
 template <int NTH>
-__global__ void __launch_bounds__(NTH, 1024 / NTH) cover_kernel(Problem P, Buffers bf) {
+__global__ void __launch_bounds__(NTH, 1024 / NTH) cover_kernel(const __grid_constant__ Problem P, const __grid_constant__ Buffers bf) {
+  dependent_start();
   extern __shared__ uint32_t dyn[];
   uint32_t* hist = dyn;
   uint32_t* cand = dyn + hist_words<NTH, true>();   // kCoverCand keys, then their indices
@@ -1185,9 +1186,10 @@ __device__ bool select_kept_fine(const uint32_t* keys, int n, int keep, int32_t*
 // from_scores: S comes from bf.scores as given; otherwise it is built here.
 // NT threads per CTA (512, or 1024 when the units are fewer than the SMs).
 template <int NT>
-__global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(Problem P, Buffers bf, int32_t* out_idx,
+__global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(const __grid_constant__ Problem P,
+                                                     const __grid_constant__ Buffers bf, int32_t* out_idx,
                                                      int from_scores, int staged_cap) {
-  constexpr int NW = NT / 32;
+  dependent_start();
   extern __shared__ uint32_t dyn[];
   uint32_t* hist = dyn;
   uint32_t* cand = dyn + hist_words<NT, false>();     // kTopkCand first-digit candidates
@@ -1376,7 +1378,8 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(Problem P,
 }
 
 // mass[l][h][t] = sum over g (ascending) of gmass[l][h][g][t].
-__global__ void mass_sum_kernel(Problem P, Buffers bf) {
+__global__ void mass_sum_kernel(const __grid_constant__ Problem P, const __grid_constant__ Buffers bf) {
+  dependent_start();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int h = blockIdx.y, l = blockIdx.z;
   if (t >= P.total_T) return;
@@ -1387,9 +1390,11 @@ __global__ void mass_sum_kernel(Problem P, Buffers bf) {
 
 // One output row (c, h) per group of 16-byte lanes.
 template <int ROWB>
-__global__ void __launch_bounds__(256) gather_kernel(Problem P, Buffers bf, const uint8_t* K,
-                                                     const uint8_t* V, const int32_t* idx,
-                                                     uint8_t* oK, uint8_t* oV) {
+__global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Problem P,
+                                                     const __grid_constant__ Buffers bf,
+                                                     const uint8_t* K, const uint8_t* V,
+                                                     const int32_t* idx, uint8_t* oK, uint8_t* oV) {
+  dependent_start();
   constexpr int LPR = ROWB / 16;  // lanes per row
   const int l = blockIdx.y;
   const long long q = (long long)blockIdx.x * (256 / LPR) + threadIdx.x / LPR;
@@ -1420,8 +1425,7 @@ __global__ void __launch_bounds__(256) gather_kernel(Problem P, Buffers bf, cons
 cudaError_t launch_mass_sum(const Problem& P, const Buffers& bf, cudaStream_t st) {
   if (!bf.mass || P.total_T == 0) return cudaSuccess;
   dim3 grid((P.total_T + 255) / 256, P.Hkv, P.L);
-  mass_sum_kernel<<<grid, 256, 0, st>>>(P, bf);
-  return cudaGetLastError();
+  return launch_kernel(mass_sum_kernel, grid, 256, 0, st, P.overlap, 0, P, bf);
 }
 
 cudaError_t launch_cover(const Problem& P, const Buffers& bf, cudaStream_t st) {
@@ -1441,8 +1445,7 @@ cudaError_t launch_cover(const Problem& P, const Buffers& bf, cudaStream_t st) {
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != \
         cudaSuccess)                                                                         \
       return e;                                                                              \
-    cover_kernel<NTH><<<grid, NTH, smem, st>>>(P, bf);                                       \
-    return cudaGetLastError();                                                               \
+    return launch_kernel(cover_kernel<NTH>, grid, NTH, smem, st, P.overlap, 0, P, bf);        \
   }
   if (units <= 2LL * nsm) MMSHIFT_COVER(512)
   MMSHIFT_COVER(256)
@@ -1466,8 +1469,8 @@ cudaError_t launch_topk(const Problem& P, const Buffers& bf, cudaStream_t st, in
     if ((e = cudaFuncSetAttribute(topk_kernel<NTT>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
                                   (int)smem)) != cudaSuccess)                                   \
       return e;                                                                                 \
-    topk_kernel<NTT><<<grid, NTT, smem, st>>>(P, bf, out_idx, from_scores ? 1 : 0, staged);      \
-    return cudaGetLastError();                                                                  \
+    return launch_kernel(topk_kernel<NTT>, grid, NTT, smem, st, P.overlap, 0, P, bf, out_idx,     \
+                         from_scores ? 1 : 0, staged);                                          \
   }
   if (units <= nsm) MMSHIFT_TOPK(1024)
   MMSHIFT_TOPK(512)
@@ -1483,9 +1486,9 @@ cudaError_t launch_gather(const Problem& P, const Buffers& bf, cudaStream_t st, 
   {                                                                                          \
     constexpr int LPR = RB / 16;                                                             \
     dim3 grid((unsigned)((rows + (256 / LPR) - 1) / (256 / LPR)), P.L);                      \
-    gather_kernel<RB><<<grid, 256, 0, st>>>(P, bf, (const uint8_t*)K, (const uint8_t*)V, idx, \
-                                            (uint8_t*)outK, (uint8_t*)outV);                 \
-    return cudaGetLastError();                                                               \
+    return launch_kernel(gather_kernel<RB>, grid, 256, 0, st, P.overlap, 0, P, bf,            \
+                         (const uint8_t*)K, (const uint8_t*)V, idx, (uint8_t*)outK,          \
+                         (uint8_t*)outV);                                                    \
   }
   switch (rowb) {
     case 128: MMSHIFT_GATHER(128)
