@@ -32,6 +32,10 @@ struct ReqInfo {
   int32_t word_off;  // offset of the request in a coverage bitmap row (32-bit words)
   int32_t split_off; // first key split of the request in the softmax partials
   int32_t nsplit;    // key splits of the request
+  // coverage vote: keys at or above cover_key (weight cover_spec in 2^-40 units)
+  // are collected in the pass that forms the total; 0 and ~0 collect none
+  uint32_t cover_key;
+  uint64_t cover_spec;
 };
 
 // Everything a kernel needs to know about one call, passed by value.
