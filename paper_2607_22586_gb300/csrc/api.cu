@@ -64,12 +64,6 @@ mmshift_status check_params(const mmshift_params* p) {
   return MMSHIFT_OK;
 }
 
-// Key split length of the softmax pass. It is a constant, so the order in
-// which a request's partial (max, sum) pairs are merged -- and with it every
-// bit of the result -- does not depend on the other requests or layers of the
-// call.
-constexpr int kSplitLen = 1024;
-
 mmshift_status build_problem(const mmshift_shape* s, const mmshift_params* p, Problem* P) {
   std::memset(P, 0, sizeof(*P));
   P->B = s->batch;

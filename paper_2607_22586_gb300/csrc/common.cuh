@@ -14,6 +14,11 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kChunk = 16;       // proxy rows per packing chunk (one group id)
 constexpr int kRowTile = 256;    // proxy rows are padded to a multiple of this
 constexpr int kMaxSplitAnchor = 8;  // anchor_split needs r <= this (one warp per anchor row)
+// Key split length of the softmax pass. It is a constant, so the order in
+// which a request's partial (max, sum) pairs are merged -- and with it every
+// bit of the result -- does not depend on the other requests or layers of the
+// call.
+constexpr int kSplitLen = 1024;
 constexpr int kUmmaPartSlots = 4; // softmax partials per (row, split) of the tensor-core pass
 
 // Status bits the kernels OR into the workspace status word.

@@ -867,8 +867,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 // ---------------------------------------------------------------- anchor rows (anchor_split)
 // The anchor is the last window query's attention over the request's keys,
 // averaged over the r query heads of the KV head (Section 3.2.3). With
-// anchor_split the mass pass writes its logits (alog, log2 units). Then, per
-// (key split, KV head, layer): anchor_part_kernel takes each anchor row's
+// anchor_split the mass pass writes its logits (alog, log2 units). Then
+// anchor_kernel (below) or, for longer requests, two kernels, per (key split,
+// KV head, layer): anchor_part_kernel takes each anchor row's
 // (max, sum of exp2(y - max)) over the split's keys (apart), and
 // anchor_final_kernel merges the request's partials in split order into c_j =
 // log2 sum_t exp2(y_jt) and writes anchor_t = (sum_j exp2(y_jt - c_j)) / r
@@ -977,6 +978,103 @@ __global__ void __launch_bounds__(ANT) anchor_final_kernel(const __grid_constant
     }
   }
 }
+
+// Both kernels in one, for batches whose longest request has at most kFusedSplits
+// key splits: a cluster of cs CTAs, one per split, for each (layer, request, KV
+// head). A CTA keeps its split's logits in registers between the two steps (warp
+// j: anchor row j, 32 keys per lane), so they are read once and there is one
+// launch instead of two; the partials go through the cluster's shared memory. The
+// order of every sum is that of the two kernels. One layer of 4096 keys 10.7 ->
+// 8.4 us, 28 layers of 8K keys 21.0 -> 16.6 us. Longer requests, as 2 to 4 splits
+// per CTA of the largest portable cluster, lose more to the registers than the
+// second read costs (28 layers of 32K keys 52 -> 90 us, ten layers of the
+// 72B-class batch 89 -> 125 us): they keep the two kernels.
+constexpr int kFusedSplits = 8;
+
+__global__ void __launch_bounds__(ANT) anchor_kernel(const __grid_constant__ Problem P,
+                                                     const __grid_constant__ Buffers bf, int cs) {
+  dependent_start();
+  static_assert(kSplitLen % (8 * 32) == 0 && kSplitLen % ANT == 0, "a split in whole runs");
+  constexpr int U = 8, NR = kSplitLen / (U * 32);   // keys per lane: NR runs of U
+  __shared__ float2 part[kMaxSplitAnchor];
+  __shared__ float buf[kMaxSplitAnchor][kSplitLen];
+  const int b = blockIdx.x / cs, s = blockIdx.x % cs, h = blockIdx.y, l = blockIdx.z;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int t0 = s * kSplitLen, t_len = P.req[b].t_len, tok_off = P.req[b].tok_off, ns = P.req[b].nsplit;
+  float v[NR][U];
+  if (w < P.r) {
+    const float* y = bf.alog + (((size_t)l * P.Hkv + h) * P.r + w) * P.total_T + tok_off;
+#pragma unroll
+    for (int q = 0; q < NR; ++q)
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int t = t0 + (q * U + u) * 32 + lane;
+        v[q][u] = t < t_len ? __ldg(y + t) : -INFINITY;
+      }
+    float m = -INFINITY, z = 0.f;
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+      float cm = v[q][0];
+#pragma unroll
+      for (int u = 1; u < U; ++u) cm = fmaxf(cm, v[q][u]);
+      if (cm == -INFINITY) continue;
+      if (cm > m) {
+        z *= fast_exp2(m - cm);       // 0 while m is still -inf
+        m = cm;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) z += fast_exp2(v[q][u] - m);
+    }
+    for (int off = 16; off; off >>= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
+      const float z2 = __shfl_xor_sync(0xffffffffu, z, off);
+      merge_ms(m, z, m2, z2);
+    }
+    if (lane == 0) part[w] = make_float2(m, z);
+  }
+  __syncwarp();
+  cluster_sync();
+  float c = 0.f;
+  if (w < P.r) {
+    float m = -INFINITY, z = 0.f;
+    if (lane < ns) {
+      const float2 x = ld_cluster_f2(mapa(smem_u32(&part[w]), (uint32_t)lane));
+      merge_ms(m, z, x.x, x.y);
+    }
+    for (int off = 16; off; off >>= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, m, off);
+      const float z2 = __shfl_xor_sync(0xffffffffu, z, off);
+      merge_ms(m, z, m2, z2);
+    }
+    c = __shfl_sync(0xffffffffu, m + __log2f(z), 0);
+  }
+  cluster_arrive();                    // this thread has read the others' partials
+  if (s < ns) {                        // shorter requests leave CTAs of their cluster idle
+    if (w < P.r) {
+#pragma unroll
+      for (int q = 0; q < NR; ++q)
+#pragma unroll
+        for (int u = 0; u < U; ++u) buf[w][(q * U + u) * 32 + lane] = fast_exp2(v[q][u] - c);
+    }
+    __syncthreads();
+    float* out = bf.anchor + ((size_t)l * P.Hkv + h) * P.total_T + tok_off;
+#pragma unroll
+    for (int i = 0; i < kSplitLen / ANT; ++i) {
+      const int t = i * ANT + tid;
+      float sm = 0.f;
+      for (int j = 0; j < P.r; ++j) sm += buf[j][t];
+      if (t0 + t < t_len) out[t0 + t] = sm / (float)P.r;
+    }
+  }
+  cluster_wait();                      // the others have read this CTA's
+}
+
+int max_splits(const Problem& P) {
+  int n = 0;
+  for (int b = 0; b < P.B; ++b) n = std::max(n, P.req[b].nsplit);
+  return n;
+}
+bool anchor_fused(const Problem& P) { return max_splits(P) <= kFusedSplits; }
 
 // ---------------------------------------------------------------- host side
 Sched make_sched(const Problem& P, int pass) {
@@ -1141,12 +1239,16 @@ bool umma_supported(const Problem& P) {
   return P.RG <= SROWS && P.anchor_rows <= SROWS && umma_softmax_supported(P);
 }
 
-int umma_launches(const Problem& P) { return P.anchor_split ? 5 : 3; }
+int umma_launches(const Problem& P) { return P.anchor_split ? (anchor_fused(P) ? 4 : 5) : 3; }
 
 // The anchor rows of an anchor_split call, after the mass pass (their own
 // stage, so that the mass pass is timed alone).
 cudaError_t launch_anchor_split(const Problem& P, const Buffers& bf, cudaStream_t st) {
   if (!P.anchor_split || !P.total_T) return cudaSuccess;
+  if (anchor_fused(P)) {
+    const int cs = max_splits(P);
+    return launch_kernel(anchor_kernel, dim3(P.B * cs, P.Hkv, P.L), ANT, 0, st, P.overlap, cs, P, bf, cs);
+  }
   const dim3 grid(P.total_splits, P.Hkv, P.L);
   const cudaError_t e = launch_kernel(anchor_part_kernel, grid, ANT, 0, st, P.overlap, 0, P, bf);
   if (e != cudaSuccess) return e;
