@@ -126,14 +126,65 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x) {
   return x;
 }
 
+// Sum of the first w warps' counts, by a whole warp (w < 32).
+__device__ __forceinline__ unsigned warps_before(const unsigned* cnt, int w) {
+  const int lane = threadIdx.x & 31;
+  return __reduce_add_sync(0xffffffffu, lane < w ? cnt[lane] : 0u);
+}
+
+// Rank of candidate c in (key desc, index asc) order of (key, idx)[0, nc), nc <=
+// NTH, for the first of the 2^tl threads that share a candidate (their c is the
+// same; ~0 for all others). They count the larger keys, four to a 16-byte read
+// and two instructions each; comparing key << 32 | ~index took four and a read of
+// its own (329 candidates of 1024 keys: 10,300 clocks of the vote's 15,900, bound
+// by instruction issue). Candidates that find others at their rank then count
+// the equal keys of lower index. `cnt` holds NTH words; `key` has room for NTH
+// keys, is 16-byte aligned and is padded with zeros, below every key. The caller's
+// barrier precedes it.
+template <int NTH>
+__device__ __forceinline__ unsigned rank_among(uint32_t* key, const uint32_t* idx, int nc,
+                                               unsigned* cnt, int& c) {
+  const int tid = threadIdx.x;
+  int tl = 0;
+  while (tl < 5 && (nc << (tl + 1)) <= NTH) ++tl;
+  const int step = 1 << tl, sub = tid & (step - 1), n4 = (nc + 3) >> 2;
+  c = tid >> tl;
+  if (tid < nc) cnt[tid] = 0u;
+  if (tid >= nc && tid < 4 * n4) key[tid] = 0u;
+  __syncthreads();
+  const bool live = c < nc;
+  const uint32_t me = live ? key[c] : 0xFFFFFFFFu;
+  const uint4* key4 = reinterpret_cast<const uint4*>(key);
+  unsigned rank = 0;
+  if (live) {
+#pragma unroll 4
+    for (int e = sub; e < n4; e += step) {
+      const uint4 y = key4[e];
+      rank += (y.x > me ? 1u : 0u) + (y.y > me ? 1u : 0u);
+      rank += (y.z > me ? 1u : 0u) + (y.w > me ? 1u : 0u);
+    }
+  }
+  for (int off = 1; off < step; off <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, off);
+  const bool first = live && sub == 0;
+  if (first) atomicAdd(&cnt[rank], 1u);
+  __syncthreads();
+  if (!first) return 0xFFFFFFFFu;
+  if (cnt[rank] > 1u) {
+    const uint32_t ix = idx[c];
+    unsigned before = 0;
+    for (int e = 0; e < nc; ++e) before += key[e] == me && idx[e] < ix ? 1u : 0u;
+    rank += before;
+  }
+  return rank;
+}
+
 // Block-wide exclusive scan of one unsigned per warp (warp totals in S.wcnt).
 template <int NTH>
 __device__ __forceinline__ unsigned warp_excl_prefix(SelShared<NTH>& S, unsigned mine) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) S.wcnt[w] = mine;
   __syncthreads();
-  unsigned before = 0;
-  for (int i = 0; i < w; ++i) before += S.wcnt[i];
+  const unsigned before = warps_before(S.wcnt, w);
   __syncthreads();
   return before;
 }
@@ -652,39 +703,22 @@ __device__ int compact_above(const float* m, int n, uint32_t klb, uint32_t* cand
 // others by as many threads as the CTA has for it, and a scan of the weights in
 // rank order finds the last one. (One thread per candidate adding up the 64-bit
 // weights before it as it compares took 11,700 clocks for 317 candidates, of
-// the vote's 19,500 on 1024 keys. With this and the bounds taken once per call,
-// vote of one float32 layer of 1024 keys 18.4 -> 14.2 us, of the 28-layer 32K
-// stack 121 -> 106 us.) More: the remaining digit passes among them, then the
-// keys equal to the last key theta by index.
+// the vote's 19,500 on 1024 keys. With this, the bounds taken once per call and
+// rank_among: vote of one float32 layer of 1024 keys 18.4 -> 12.3 us, of the
+// 28-layer 32K stack 121 -> 102 us.) More: the remaining digit passes among
+// them, then the keys equal to the last key theta by index.
 template <int NTH>
-__device__ void cover_among(const uint32_t* cand, const uint32_t* cidx, int nc, int p0,
+__device__ void cover_among(uint32_t* cand, const uint32_t* cidx, int nc, int p0,
                             uint32_t prefix, unsigned long long target_w, int shift, float tau,
                             SelShared<NTH>& S, uint32_t* hist, uint32_t* bits) {
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   if (nc <= NTH) {
-    // key << 32 | ~index per candidate: larger ranks earlier
-    unsigned long long* comp = reinterpret_cast<unsigned long long*>(hist);
-    unsigned long long* byrank = comp + NTH;   // weights in rank order
-    if (tid == 0) S.rend = 0xFFFFFFFFu;
-    if (tid < nc) comp[tid] = ((unsigned long long)cand[tid] << 32) | (uint32_t)~cidx[tid];
-    __syncthreads();
-    int tl = 0;                                // 2^tl threads per candidate
-    while (tl < 5 && (nc << (tl + 1)) <= NTH) ++tl;
-    const int step = 1 << tl, c = tid >> tl, sub = tid & (step - 1);
-    const bool live = c < nc;
-    const unsigned long long me = live ? comp[c] : ~0ull;
-    unsigned rank = 0;
-    if (live) {
-      int e = sub;
-      for (; e + 3 * step < nc; e += 4 * step) {
-        const unsigned long long y0 = comp[e], y1 = comp[e + step], y2 = comp[e + 2 * step],
-                                 y3 = comp[e + 3 * step];
-        rank += (y0 > me) + (y1 > me) + (y2 > me) + (y3 > me);
-      }
-      for (; e < nc; e += step) rank += comp[e] > me;
-    }
-    for (int off = 1; off < step; off <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, off);
-    if (live && sub == 0) byrank[rank] = fx_weight((uint32_t)(me >> 32), shift);
+    unsigned long long* byrank = reinterpret_cast<unsigned long long*>(hist);   // weights in rank order
+    if (tid == 0) S.rend = 0xFFFFFFFEu;
+    int c;
+    const unsigned rank =
+        rank_among<NTH>(cand, cidx, nc, reinterpret_cast<unsigned*>(byrank + NTH), c);
+    if (rank != 0xFFFFFFFFu) byrank[rank] = fx_weight(cand[c], shift);
     __syncthreads();
     unsigned long long sum = tid < nc ? byrank[tid] : 0ull;
     for (int off = 1; off < 32; off <<= 1) {
@@ -699,8 +733,8 @@ __device__ void cover_among(const uint32_t* cand, const uint32_t* cidx, int nc, 
       if (sum >= target_w) atomicMin(&S.rend, (unsigned)tid);
     }
     __syncthreads();
-    if (live && sub == 0 && rank <= S.rend) {
-      const uint32_t ix = ~(uint32_t)me;
+    if (rank <= S.rend) {
+      const uint32_t ix = cidx[c];
       atomicOr(bits + (ix >> 5), 1u << (ix & 31));
     }
     return;
@@ -1043,7 +1077,7 @@ __device__ bool select_kept_fine(const uint32_t* keys, int n, int keep, int32_t*
   }
   if (lane == 31) S.wcnt[w] = incl;
   __syncthreads();
-  for (int i = 0; i < w; ++i) incl += S.wcnt[i];
+  incl += warps_before(S.wcnt, w);
   const unsigned excl = incl - c;
   if (excl < k && incl >= k) {
     unsigned cum = excl;
@@ -1159,8 +1193,7 @@ __device__ bool select_kept_fine(const uint32_t* keys, int n, int keep, int32_t*
   }
   if (lane == 0) S.wcnt[w] = wtot;
   __syncthreads();
-  unsigned pos = 0;
-  for (int i = 0; i < w; ++i) pos += S.wcnt[i];
+  unsigned pos = warps_before(S.wcnt, w);
   // the kept indices go to shared memory (the histograms' room) in order,
   // then out in one coalesced sweep; directly when they do not fit
   int32_t* staging = reinterpret_cast<int32_t*>(hist);
@@ -1311,7 +1344,8 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(const __gr
               word[u] = (g < P.G && base < n) ? __ldg(bw + (size_t)g * P.total_words + (base >> 5)) : 0u;
             }
 #pragma unroll
-            for (int u = 0; u < UB; ++u) vote[u] += __popc(warp_transpose32(word[u]));
+            for (int u = 0; u < UB; ++u)
+              if (base0 + u * NT < n) vote[u] += __popc(warp_transpose32(word[u]));
           }
         }
 #pragma unroll
