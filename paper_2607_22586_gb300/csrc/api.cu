@@ -149,7 +149,7 @@ Layout layout_of(const Problem& P) {
   w.scores = o; o += align256(L * P.Hkv * (size_t)P.total_T * sizeof(float));
   // count word, the list of proxy elements to recompute in float64, then the
   // exact window sums they are recomputed from
-  w.refine = o; o += 256 + align256((size_t)proxy_refine_capacity(P) * sizeof(int4));
+  w.refine = o; o += 256 + align256(proxy_refine_bytes(P));
   w.refine_stats = o; o += align256(L * P.B * P.Hq * (size_t)5 * P.d * sizeof(float));
   w.total = o;
   return w;
@@ -171,10 +171,7 @@ mmshift_status carve(const Problem& P, void* ws, size_t bytes, Buffers* bf) {
   bf->apart = reinterpret_cast<float2*>(base + w.apart);
   bf->bits = reinterpret_cast<uint32_t*>(base + w.bits);
   bf->scores = reinterpret_cast<float*>(base + w.scores);
-  bf->refine_count = reinterpret_cast<int*>(base + w.refine);
-  bf->refine_items = reinterpret_cast<int4*>(base + w.refine + 256);
-  bf->refine_cap = (int32_t)proxy_refine_capacity(P);
-  bf->refine_stats = reinterpret_cast<float*>(base + w.refine_stats);
+  set_refine_list(P, base + w.refine, reinterpret_cast<float*>(base + w.refine_stats), bf);
   return MMSHIFT_OK;
 }
 

@@ -103,12 +103,13 @@ struct Buffers {
   const int32_t* kept_len;    // [L][B][Hkv]
   // bf16 proxies whose float32 value lies too close to a rounding boundary
   // are recomputed in float64 (proxy.cu): the sampler appends them here and a
-  // second kernel redoes them; without a list (null) the sampler redoes them
-  // itself
+  // second kernel redoes them; without a list (null) it redoes every element
   int* refine_count;          // entries appended (may exceed refine_cap)
-  int4* refine_items;         // [refine_cap] (layer * B + request, query head, proxy, dim)
+  uint32_t* refine_items;     // [refine_cap] (layer * B + request, query head, proxy * d + dim), packed
   float* refine_stats;        // [L][B][Hq][5][d] exact window sums (x0, S1 hi / lo, S2 hi / lo)
   int32_t refine_cap;
+  int32_t refine_hq_bit, refine_lb_bit;   // first bits of an entry's first two fields
+  int32_t refine_wide;        // entries are 64-bit
 };
 
 // Whole-prefill statistics job (stats.cu).
@@ -239,9 +240,11 @@ cudaError_t launch_prefill_stats(const StatsJob& J, const void* Q, float* part, 
                                  cudaStream_t st, bool bf16);
 cudaError_t launch_proxy_pack(const Problem& P, const Buffers& bf, cudaStream_t st,
                               const void* qwin);
-// Proxy elements the list of bf holds for a call's shape: at most this many
-// are refined by the second kernel, the rest by the sampler itself.
-int64_t proxy_refine_capacity(const Problem& P);
+// The refinement list of a call: its bytes in the workspace, and where it lies
+// (256 bytes for the count, then the entries; a call with more undecided elements
+// than entries has all of them recomputed).
+size_t proxy_refine_bytes(const Problem& P);
+void set_refine_list(const Problem& P, char* count, float* stats, Buffers* bf);
 // Kernels launch_proxy_pack enqueues for P and bf.
 int proxy_launches(const Problem& P, const Buffers& bf);
 // ev (nullable): stage events 1 (softmax pass), 2 (merge) and 3 (mass pass)

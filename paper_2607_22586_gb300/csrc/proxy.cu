@@ -16,7 +16,7 @@
 // mu + gamma * sigma * z, rotated: the float32 evaluation is within a bound
 // of that value (2^-20 of the magnitudes involved, 2^-19 rotated; below), so
 // it rounds to the same bf16 unless a rounding boundary lies within the bound.
-// Such elements (about four in ten thousand) are recomputed in float64 -- the
+// Such elements (0.07 % at gamma = 10, 0.57 % rotated) are recomputed in float64 -- the
 // window statistics from their exact sums, the normal (log, sin, cos of the
 // same 24-bit uniforms), the sum and the rotation -- and rounded from there by
 // refine_kernel, from a list in the workspace. A call without a workspace
@@ -184,18 +184,70 @@ __device__ __forceinline__ double uniform_f64(uint32_t w) {
   return ((double)(w >> 9) + 0.5) * 1.1920928955078125e-07;
 }
 
+// Proxy element (request b of call layer l, query head hq, proxy i, dim dd)
+// before rotation, in float64: mu + (gamma sigma) z with z from the same
+// Philox words as the float32 path.
+template <int D>
+__device__ double proxy_f64(const Problem& P, const float* rs, const __nv_bfloat16* qwin, int l,
+                            int b, int hq, int i, int dd) {
+  double mu, sig;
+  win_stats_f64<D>(P, rs, qwin, l, b, hq, dd, mu, sig);
+  const int k = dd < D / 2 ? dd % 4 : 4 + (dd - D / 2) % 4;   // normal k of the draw
+  const uint64_t w64 = philox_word<D>(P, l, b, hq, i, (dd % (D / 2)) / 4, k);
+  const double u2 = uniform_f64((uint32_t)(w64 >> 32));
+  const double rad = sqrt(-2.0 * log(uniform_f64((uint32_t)w64)));
+  const double z = __dmul_rn(rad, (k & 1) ? sinpi(2.0 * u2) : cospi(2.0 * u2));
+  return __dadd_rn(mu, __dmul_rn(__dmul_rn((double)P.gamma, sig), z));
+}
+
+// The rotation angle of RoPE pair f of request b: its sine and cosine in float64.
+template <int D>
+__device__ __forceinline__ void rotation_f64(const Problem& P, int b, int f, double& sn, double& cs) {
+  const double pos = (double)(P.req[b].t_len + P.rope_off);
+  sincos(pos * pow((double)P.rope_theta, -2.0 * f / (double)D), &sn, &cs);
+}
+
+// Stores the bf16 rounding of element (l, b, hq, i, dd) into the packed block
+// and the caller-layout copy.
+template <int D>
+__device__ __forceinline__ void store_refined(const Problem& P, const Buffers& bf, int l, int b,
+                                              int hq, int i, int dd, double v) {
+  const __nv_bfloat16 o = __double2bfloat16(v);
+  const int h = hq / P.r, j = hq - h * P.r;
+  if (bf.packed) {
+    __nv_bfloat16* packed = (__nv_bfloat16*)bf.packed +
+                            ((((size_t)l * P.B + b) * P.Hkv + h) * P.Prows_pad) * D;
+    packed[packed_row(P, i, j) * D + dd] = o;
+  }
+  if (bf.proxies_out)
+    ((__nv_bfloat16*)bf.proxies_out)[((((size_t)l * P.B + b) * P.Hq + hq) * P.Np + i) * D + dd] = o;
+}
+
+// A list entry: layer * B + request, query head, proxy and dimension side by
+// side, each in as many bits as it needs (set_refine_list); 64-bit where they
+// exceed 32.
+int bits_for(int64_t n) {   // values 0 .. n - 1
+  int k = 0;
+  while (((int64_t)1 << k) < n) ++k;
+  return k;
+}
+
 // Appends the undecided elements (bit k: element k of the thread's draw) of
-// proxy i to the refinement list. The count keeps growing past the list's
-// capacity, which tells refine_kernel to redo the whole call.
+// proxy i to the refinement list, with one atomic for the thread's. The count
+// keeps growing past the list's capacity, which tells refine_kernel to redo the
+// whole call.
 template <int D>
 __device__ __noinline__ void enlist(const Problem& P, const Buffers& bf, int l, int b, int hq,
                                     int i, int qq, uint32_t undecided) {
-  while (undecided) {
+  int slot = atomicAdd(bf.refine_count, __popc(undecided));
+  const uint64_t e0 = ((uint64_t)(l * P.B + b) << bf.refine_lb_bit) |
+                      ((uint64_t)hq << bf.refine_hq_bit) | (uint64_t)(i * D);
+  for (; undecided && slot < bf.refine_cap; ++slot) {
     const int k = __ffs(undecided) - 1;
     undecided &= undecided - 1;
-    const int dd = k < 4 ? 4 * qq + k : D / 2 + 4 * qq + (k - 4);
-    const int slot = atomicAdd(bf.refine_count, 1);
-    if (slot < bf.refine_cap) bf.refine_items[slot] = make_int4(l * P.B + b, hq, i, dd);
+    const uint64_t e = e0 | (k < 4 ? 4 * qq + k : D / 2 + 4 * qq + (k - 4));
+    if (bf.refine_wide) reinterpret_cast<uint64_t*>(bf.refine_items)[slot] = e;
+    else bf.refine_items[slot] = (uint32_t)e;
   }
 }
 
@@ -365,6 +417,40 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
   }
 }
 
+// Every element of a call without a list, recomputed in float64: one thread per
+// element or rotated pair. All float64 units are busy, so the parts of an element
+// side by side (refine_kernel) would only wait for one another: 28 heads, N = 512,
+// rotated, 2,541 us with one thread per element, 2,574 us side by side, 1,294 us
+// with one thread per pair.
+template <int D>
+__global__ void __launch_bounds__(128) refine_all_kernel(const __grid_constant__ Problem P,
+                                                         const __grid_constant__ Buffers bf,
+                                                         const __nv_bfloat16* qwin) {
+  dependent_start();
+  constexpr int half = D / 2;
+  const bool rope = P.rope_theta > 0.f;
+  const int64_t n = (int64_t)P.L * P.B * P.Hq * P.Np * (rope ? half : D);
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
+    const int per = rope ? half : D;
+    const int f = (int)(e % per);
+    uint32_t q = (uint32_t)(e / per);        // 2^32 rows would be 550 GB of proxies
+    const int i = (int)(q % (uint32_t)P.Np); q /= (uint32_t)P.Np;
+    const int hq = (int)(q % (uint32_t)P.Hq); q /= (uint32_t)P.Hq;
+    const int b = (int)(q % (uint32_t)P.B), l = (int)(q / (uint32_t)P.B);
+    const double a = proxy_f64<D>(P, bf.refine_stats, qwin, l, b, hq, i, f);
+    if (!rope) {
+      store_refined<D>(P, bf, l, b, hq, i, f, a);
+      continue;
+    }
+    const double c = proxy_f64<D>(P, bf.refine_stats, qwin, l, b, hq, i, f + half);
+    double sn, cs;
+    rotation_f64<D>(P, b, f, sn, cs);
+    store_refined<D>(P, bf, l, b, hq, i, f, __dadd_rn(__dmul_rn(a, cs), -__dmul_rn(c, sn)));
+    store_refined<D>(P, bf, l, b, hq, i, f + half, __dadd_rn(__dmul_rn(c, cs), __dmul_rn(a, sn)));
+  }
+}
+
 // Elements the sampler found undecided, recomputed in float64: mu + (gamma
 // sigma) z from the same Philox words, rotated, rounded to bf16 into the packed
 // block and the caller-layout copy. A CTA takes 32 elements at a time, one warp
@@ -373,37 +459,33 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
 // angle: the time of a short call is one element's chain of float64 divisions,
 // logarithm and sine, which the warps run side by side (against one thread per
 // element, proxy stage of one layer of 28 heads, N = 512: 30.1 -> 25.8 us, of the
-// 28-layer 32K stack with few proxies 42.0 -> 33.7 us). A call whose entries overflowed the list, or that has
-// no list (all = true), has every element recomputed.
+// 28-layer 32K stack with few proxies 42.0 -> 33.7 us). A call whose entries
+// overflowed the list has every element recomputed.
 template <int D>
 __global__ void __launch_bounds__(224) refine_kernel(const __grid_constant__ Problem P,
                                                      const __grid_constant__ Buffers bf,
-                                                     const __nv_bfloat16* qwin, bool all) {
+                                                     const __nv_bfloat16* qwin) {
   dependent_start();
   __shared__ double mu[2][32], sig[2][32], rad[2][32], trig[2][32], rot[2][32];
   constexpr int half = D / 2;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const bool rope = P.rope_theta > 0.f;
-  bool list = false;
-  int64_t n = (int64_t)P.L * P.B * P.Hq * P.Np * D;
-  if (!all) {
-    const int cnt = *bf.refine_count;
-    if (cnt <= bf.refine_cap) {
-      list = true;
-      n = cnt;
-    }
-  }
+  const int cnt = *bf.refine_count;
+  const bool list = cnt <= bf.refine_cap;
+  const int64_t n = list ? cnt : (int64_t)P.L * P.B * P.Hq * P.Np * D;
   for (int64_t base = (int64_t)blockIdx.x * 32; base < n; base += (int64_t)gridDim.x * 32) {
     const int64_t e = base + lane;
     int l = 0, b = 0, hq = 0, i = 0, dd = 0;
     if (e < n) {
       if (list) {
-        const int4 it = bf.refine_items[e];
-        l = it.x / P.B;
-        b = it.x - l * P.B;
-        hq = it.y;
-        i = it.z;
-        dd = it.w;
+        const uint64_t it = bf.refine_wide ? reinterpret_cast<const uint64_t*>(bf.refine_items)[e]
+                                           : (uint64_t)bf.refine_items[e];
+        const int lb = (int)(it >> bf.refine_lb_bit);
+        l = lb / P.B;
+        b = lb - l * P.B;
+        hq = (int)((uint32_t)(it >> bf.refine_hq_bit) & ((1u << (bf.refine_lb_bit - bf.refine_hq_bit)) - 1u));
+        i = (int)((uint32_t)it & ((1u << bf.refine_hq_bit) - 1u)) / D;
+        dd = (int)((uint32_t)it % D);
       } else {
         int64_t r = e;
         dd = (int)(r % D); r /= D;
@@ -429,9 +511,7 @@ __global__ void __launch_bounds__(224) refine_kernel(const __grid_constant__ Pro
           trig[c][lane] = (k & 1) ? sinpi(2.0 * u2) : cospi(2.0 * u2);
         }
       } else {
-        const double pos = (double)(P.req[b].t_len + P.rope_off);
-        const double ang = pos * pow((double)P.rope_theta, -2.0 * f / (double)D);
-        sincos(ang, &rot[0][lane], &rot[1][lane]);
+        rotation_f64<D>(P, b, f, rot[0][lane], rot[1][lane]);
       }
     }
     __syncthreads();
@@ -446,15 +526,7 @@ __global__ void __launch_bounds__(224) refine_kernel(const __grid_constant__ Pro
         v = dd < half ? __dadd_rn(__dmul_rn(a, cs), -__dmul_rn(c, sn))
                       : __dadd_rn(__dmul_rn(c, cs), __dmul_rn(a, sn));
       }
-      const __nv_bfloat16 o = __double2bfloat16(v);
-      const int h = hq / P.r, j = hq - h * P.r;
-      if (bf.packed) {
-        __nv_bfloat16* packed = (__nv_bfloat16*)bf.packed +
-                                ((((size_t)l * P.B + b) * P.Hkv + h) * P.Prows_pad) * D;
-        packed[packed_row(P, i, j) * D + dd] = o;
-      }
-      if (bf.proxies_out)
-        ((__nv_bfloat16*)bf.proxies_out)[((((size_t)l * P.B + b) * P.Hq + hq) * P.Np + i) * D + dd] = o;
+      store_refined<D>(P, bf, l, b, hq, i, dd, v);
     }
     __syncthreads();   // the values are used before the next elements'
   }
@@ -496,18 +568,38 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
   proxy_pack_kernel<T, D><<<grid, 256, 0, st>>>(P, b2, (const T*)qwin, nch);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (refine) {
-    const bool all = b2.refine_items == nullptr;
+    if (!b2.refine_items)
+      return launch_kernel(refine_all_kernel<D>, dim3(8 * std::max(nsm, 1)), 128, 0, st, P.overlap, 0,
+                           P, b2, (const __nv_bfloat16*)qwin);
     e = launch_kernel(refine_kernel<D>, dim3(8 * std::max(nsm, 1)), P.rope_theta > 0.f ? 224 : 96, 0,
-                      st, P.overlap, 0, P, b2, (const __nv_bfloat16*)qwin, all);
+                      st, P.overlap, 0, P, b2, (const __nv_bfloat16*)qwin);
   }
   return e;
 }
 
 }  // namespace
 
-int64_t proxy_refine_capacity(const Problem& P) {
+// 16 bytes per 256 elements and 64 KB: with 4 bytes an entry 1.56 % of them, above
+// the 0.57 % that are undecided rotated (0.92 % at gamma = 2). Entries of 16 bytes
+// (0.39 %) overflowed in rotated calls of more than two million elements, whose
+// every element was then recomputed: proxy stage of 14 layers of 32 heads, two
+// requests, N = 128, rotated, 10.3 ms -> 156 us;
+// nine layers of 16 heads, five requests, N = 32, 2,107 -> 62 us.
+size_t proxy_refine_bytes(const Problem& P) {
   const int64_t elems = (int64_t)P.L * P.B * P.Hq * P.Np * P.d;
-  return std::min<int64_t>(elems / 256 + 4096, (int64_t)1 << 30);
+  return 16 * (size_t)std::min<int64_t>(elems / 256 + 4096, (int64_t)1 << 30);
+}
+
+void set_refine_list(const Problem& P, char* count, float* stats, Buffers* bf) {
+  bf->refine_count = reinterpret_cast<int*>(count);
+  bf->refine_items = reinterpret_cast<uint32_t*>(count + 256);
+  bf->refine_stats = stats;
+  bf->refine_hq_bit = bits_for((int64_t)P.Np * P.d);   // d is a power of two
+  bf->refine_lb_bit = bf->refine_hq_bit + bits_for(P.Hq);
+  bf->refine_wide = bf->refine_lb_bit + bits_for((int64_t)P.L * P.B) > 32;
+  const size_t n = proxy_refine_bytes(P) / (bf->refine_wide ? 8 : 4);
+  bf->refine_cap = (int32_t)std::min<size_t>(n, 0x7FFFFFFF);
+  if (bf->refine_hq_bit > 31) bf->refine_cap = 0;   // 4 GB a head: no list
 }
 
 int proxy_launches(const Problem& P, const Buffers& bf) { return samples_bf16(P, bf) ? 2 : 1; }
