@@ -215,8 +215,10 @@ def measure_coverage(args, wl, shape, K, Q, out_idx, stream, seed, M, tpeak, tki
     ms = e0.elapsed_time(e1) / 3
     c = cov.flatten().double().cpu().numpy()
     cr = cov_recent.flatten().double().cpu().numpy()
-    # two passes (softmax, mass) of 2 d flops per (decode query, query head, key)
-    flops = 2 * 2.0 * wl.head_dim * n_dec * wl.n_q_heads * wl.total_tokens * L
+    # the logits of every prompt key and of the kept keys: 2 d flops per (decode
+    # query, query head, key)
+    kept = sum(min(t, c) for t, c in zip(wl.seq_lens, wl.budgets))
+    flops = 2.0 * wl.head_dim * n_dec * wl.n_q_heads * (wl.total_tokens + kept) * L
     ach = flops / (ms * 1e-3) / 1e12
     return {"n_decode_queries": n_dec, "queries": "0.5 * per-head key mean + N(0, 1.5^2), synthetic",
             "mean": float(c.mean()), "p10": float(np.percentile(c, 10)), "min": float(c.min()),
@@ -224,10 +226,10 @@ def measure_coverage(args, wl, shape, K, Q, out_idx, stream, seed, M, tpeak, tki
             "ms_per_call": ms,
             "roofline": {"bound": "tensor", "achieved": ach, "peak": tpeak, "unit": "TFLOP/s",
                          "frac": ach / tpeak, "traffic": None, "peak_kind": tkind,
-                         "kernel": "whole mmshift_coverage call (pack, softmax pass, merge, mass pass, "
-                                   "coverage)",
-                         "note": "algorithmic flops of the decode queries only; each query is its own "
-                                 "group, padded from r to 16 rows per KV head"}}
+                         "kernel": "whole mmshift_coverage call (pack, copy of the kept rows, softmax "
+                                   "pass over the prompt and over the copied rows, ratio)",
+                         "note": "algorithmic flops of the decode queries only; the r * n_dec rows of a "
+                                 "KV head are padded to blocks of 256"}}
 
 
 class PreStep:
@@ -903,7 +905,7 @@ def run_gpu(args, wl):
             extra_roofs["hidden_proxies_roofline"] = {
                 "bound": "tensor", "achieved": ach, "peak": tpeak, "unit": "TFLOP/s",
                 "frac": ach / tpeak, "traffic": None,
-                "kernel": "hidden_sample_kernel + hidden_proj_kernel",
+                "kernel": "hidden_sample_kernel + hidden_proj_pair_kernel",
                 "flops_per_launch": flops, "peak_kind": tkind}
     tokens_layer = T * L * world          # metric unit: tokens per second per layer
     value = job_value(T * L, world, ms)

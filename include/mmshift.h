@@ -339,10 +339,13 @@ mmshift_status mmshift_topk_head_budgets(const mmshift_shape* s, const float* sc
  * in [0, T_b); -1 marks padding rows and is skipped; other values are
  * skipped and reported by mmshift_poll_status) and
  * averaged over the r query heads of h: cov [L][batch][Hkv][n_dec] float32.
- * Steps 2-4 run with the decode queries as n_dec groups of one proxy (so the
- * masses come from the same kernels as the selection's); Qwin supplies the
- * anchor rows those kernels also compute. softmax_scale 0 = 1/sqrt(d);
- * 1 <= n_dec <= 1024; workspace: mmshift_coverage_workspace_size() bytes. */
+ * The kept and the whole sum of exponentials of each query head come from the
+ * selection's softmax pass, over the kept rows (copied together first) and over
+ * the prompt. Where the copied rows do not fit in the workspace, steps 2-4 run
+ * with the decode queries as n_dec groups of one proxy instead and the kept
+ * keys' masses are added up; Qwin supplies the anchor rows of that form.
+ * softmax_scale 0 = 1/sqrt(d); 1 <= n_dec <= 1024; workspace:
+ * mmshift_coverage_workspace_size() bytes. */
 mmshift_status mmshift_coverage_workspace_size(const mmshift_shape* s, int32_t n_dec,
                                                size_t* bytes);
 mmshift_status mmshift_coverage(const mmshift_shape* s, const void* K, const void* Qwin,

@@ -3,9 +3,12 @@
 // (Section 3.2.2; Appendix B). Two persistent, warp-specialised kernels of
 // 576 threads, one CTA per SM:
 //   warp 0      TMA producer (stationary proxy rows, a ring of K tiles);
-//   warp 1      TMEM allocator and MMA issuer (one thread);
+//   warp 1      TMEM allocator and MMA issuer (the whole warp waits, one
+//               elected lane issues);
 //   warps 2-17  epilogue (four warpgroups): tcgen05.ld of the accumulators,
-//               exp2 and reductions in registers, outputs to global memory.
+//               exp2 and reductions in registers, outputs to global memory;
+//               an accumulator is released as soon as its last columns are in
+//               registers.
 // Work units are (layer, request, KV head, key split of 1024 keys, proxy
 // block). Teams of one CTA (softmax: one CTA pair) per proxy block walk
 // contiguous ranges of key splits, so the team reads each K tile together
