@@ -14,9 +14,9 @@
 //
 // bf16 proxies equal the bf16 rounding of the exact (real-number) value of
 // mu + gamma * sigma * z, rotated: the float32 evaluation is within a bound
-// of that value (2^-20 of the magnitudes involved, 2^-19 rotated; below), so
+// of that value (2^-20 of the magnitudes involved; rotated, below), so
 // it rounds to the same bf16 unless a rounding boundary lies within the bound.
-// Such elements (0.07 % at gamma = 10, 0.57 % rotated) are recomputed in float64 -- the
+// Such elements (0.07 % at gamma = 10, 0.25 % rotated) are recomputed in float64 -- the
 // window statistics from their exact sums, the normal (log, sin, cos of the
 // same 24-bit uniforms), the sum and the rotation -- and rounded from there by
 // refine_kernel, from a list in the workspace. A call without a workspace
@@ -103,14 +103,23 @@ __device__ __forceinline__ void win_stats(const WinSums& w, float x0, int W, flo
   sg = sqrtf(fmaxf(var, 0.f));
 }
 
-// Bound on |float32 value - exact value| of a proxy element relative to the
-// magnitudes it is made of: |mu| + |mean - x0| + |gamma sigma z|, summed over
-// the RoPE pair when rotated. Unrotated the float32 path stays within about
-// 9 ulp of them: the normal about 4.8 (log 3, square root 0.5, sine / cosine
-// 2), sigma and gamma sigma 1.8, the mean 1, the FMA 0.5. Rotated, the
-// table's sine / cosine (2 ulp) and the rotation's roundings add about 3.5.
-constexpr float kRefineRel = 1.0f / 1048576.0f;      // 2^-20
-constexpr float kRefineRelRope = 1.0f / 524288.0f;   // 2^-19
+// Bound on |float32 value - exact value| of a proxy element. Unrotated it is
+// relative to the magnitudes m = |mu| + |mean - x0| + |gamma sigma z| it is made
+// of: the float32 path stays within about 9 ulp (2^-24) of them: the normal about
+// 4.8 (log 3, square root 0.5, sine / cosine 2), sigma and gamma sigma 1.8, the
+// mean 1, the FMA 0.5.
+//
+// Rotated by the table's cosine C and sine S, a' = a C - c S has, in ulp, 9 of
+// m_a |C| + m_c |S| from a and c; 4 of the same from the table (2 ulp of
+// relative size 2^-23); 2 of m_a |S| + m_c |C| from the angle, whose rounding to
+// float32 is at most 2^-23; and 1.5 from the products and the difference: within
+// 14.5 and 2. The bound takes 24 and 4. A bound of 32 ulp of m_a + m_c, which does
+// not tell the weights of the pair's two elements apart, left 0.57 % of the
+// elements undecided instead of 0.25 % (proxy stage of 14 layers of 32 heads, two
+// requests, N = 128: 156 -> 118 us).
+constexpr float kRefineRel = 1.0f / 1048576.0f;            // 2^-20
+constexpr float kRefineSame = 24.0f / 16777216.0f;         // 24 ulp
+constexpr float kRefineCross = 4.0f / 16777216.0f;         // 4 ulp
 
 // Whether rounding to bf16 is decided by the float32 value v within +-err
 // (both ends rounded by one paired conversion).
@@ -256,7 +265,8 @@ __device__ __noinline__ void enlist(const Problem& P, const Buffers& bf, int l, 
 // where the call would not fill the SMs (launch_t).
 constexpr int kProxyChunks = 8;
 
-template <typename T, int D>
+// ROPE: rotated proxies. As a branch at run time it cost unrotated calls 0.2 %.
+template <typename T, int D, bool ROPE>
 __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers bf, const T* qwin,
                                                          int nch) {
   dependent_start();
@@ -264,7 +274,10 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
   const int b = blockIdx.y, l = blockIdx.z;
   const int h = hq / P.r, j = hq - h * P.r;
   // mean, std, and |mean| + |mean - x0| (the mean's part of the error bound)
-  __shared__ float mu[D], sg[D], mmag[D], rc[D / 2], rs[D / 2];
+  __shared__ float mu[D], sg[D], mmag[D];
+  // the rotation, and the weights of the pair's magnitudes in the bound
+  constexpr int NR = ROPE ? D / 2 : 1;
+  __shared__ float rc[NR], rs[NR], ec[NR], es[NR];
   constexpr int RPT = 256 / D;               // threads per dimension
   __shared__ WinSums part[RPT][D];
   const T* q = qwin ? qwin + (size_t)l * P.ls_q + ((size_t)b * P.W * P.Hq + hq) * D : nullptr;
@@ -310,8 +323,7 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
       }
     }
   }
-  const bool rope = P.rope_theta > 0.f && !bf.proxies_in;
-  if (rope) {
+  if constexpr (ROPE) {
     // angle = pos * theta^(-2k/d), reduced modulo 2*pi in double once per block
     const double pos = (double)(P.req[b].t_len + P.rope_off);
     for (int k = threadIdx.x; k < D / 2; k += blockDim.x) {
@@ -320,6 +332,8 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
       float sv, cv;
       sincosf((float)red, &sv, &cv);
       rc[k] = cv; rs[k] = sv;
+      ec[k] = kRefineSame * fabsf(cv) + kRefineCross * fabsf(sv);
+      es[k] = kRefineSame * fabsf(sv) + kRefineCross * fabsf(cv);
     }
   }
   __syncthreads();
@@ -355,18 +369,22 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
         const float g0 = P.gamma * sg[d0], g1 = P.gamma * sg[d1];
         float a = fmaf(g0, z[k], mu[d0]), c = fmaf(g1, z[4 + k], mu[d1]);
         float ma = mmag[d0] + fabsf(g0 * z[k]), mc = mmag[d1] + fabsf(g1 * z[4 + k]);
-        if (rope) {
+        if constexpr (ROPE) {
           const float ar = a * rc[d0] - c * rs[d0];
           c = c * rc[d0] + a * rs[d0];
           a = ar;
-          ma = mc = ma + mc;
+          const float ea = ma * ec[d0] + mc * es[d0];
+          mc = mc * ec[d0] + ma * es[d0];
+          ma = ea;
+        } else {
+          ma *= kRefineRel;
+          mc *= kRefineRel;
         }
         v[k] = a;
         v[4 + k] = c;
-          if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-          const float rel = rope ? kRefineRelRope : kRefineRel;
-          undecided |= (bf16_undecided(a, rel * ma) ? 1u : 0u) << k;
-          undecided |= (bf16_undecided(c, rel * mc) ? 1u : 0u) << (4 + k);
+        if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+          undecided |= (bf16_undecided(a, ma) ? 1u : 0u) << k;
+          undecided |= (bf16_undecided(c, mc) ? 1u : 0u) << (4 + k);
         }
       }
       if (undecided && bf.refine_items && !bf.stats_in) enlist<D>(P, bf, l, b, hq, i, qq, undecided);
@@ -565,7 +583,10 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
       (e = cudaMemsetAsync(b2.refine_count, 0, sizeof(int), st)) != cudaSuccess)
     return e;
   dim3 grid(P.Hq * nch, P.B, P.L);
-  proxy_pack_kernel<T, D><<<grid, 256, 0, st>>>(P, b2, (const T*)qwin, nch);
+  if (P.rope_theta > 0.f && !bf.proxies_in)
+    proxy_pack_kernel<T, D, true><<<grid, 256, 0, st>>>(P, b2, (const T*)qwin, nch);
+  else
+    proxy_pack_kernel<T, D, false><<<grid, 256, 0, st>>>(P, b2, (const T*)qwin, nch);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (refine) {
     if (!b2.refine_items)
@@ -579,10 +600,10 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
 
 }  // namespace
 
-// 16 bytes per 256 elements and 64 KB: with 4 bytes an entry 1.56 % of them, above
-// the 0.57 % that are undecided rotated (0.92 % at gamma = 2). Entries of 16 bytes
-// (0.39 %) overflowed in rotated calls of more than two million elements, whose
-// every element was then recomputed: proxy stage of 14 layers of 32 heads, two
+// 16 bytes per 256 elements and 64 KB: with 4 bytes an entry 1.56 % of them, well
+// above the 0.25 % that are undecided rotated (0.4 % at gamma = 2). Entries of 16
+// bytes (0.39 %) overflowed in rotated calls of more than two million elements
+// when the bound left 0.57 %, and every element was then recomputed: proxy stage of 14 layers of 32 heads, two
 // requests, N = 128, rotated, 10.3 ms -> 156 us;
 // nine layers of 16 heads, five requests, N = 32, 2,107 -> 62 us.
 size_t proxy_refine_bytes(const Problem& P) {
