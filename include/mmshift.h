@@ -339,6 +339,8 @@ mmshift_status mmshift_topk_head_budgets(const mmshift_shape* s, const float* sc
  * in [0, T_b); -1 marks padding rows and is skipped; other values are
  * skipped and reported by mmshift_poll_status) and
  * averaged over the r query heads of h: cov [L][batch][Hkv][n_dec] float32.
+ * Where a logit of the decode query under any of these heads is NaN or +inf,
+ * or all of a head's are -inf, cov is 0, whether such a key is kept or not.
  * The kept and the whole sum of exponentials of each query head come from the
  * selection's softmax pass, over the kept rows (copied together first) and over
  * the prompt. Where the copied rows do not fit in the workspace, steps 2-4 run

@@ -152,8 +152,10 @@ __global__ void __launch_bounds__(256) ratio_kernel(const __grid_constant__ Prob
       float m = -INFINITY, z = 0.f, mk = -INFINITY, zk = 0.f;
       merged(P, all, j * P.gs + i, m, z);
       merged(Pk, kept, j * P.gs + i, mk, zk);
-      // zk 2^(mk - m) <= z, so neither factor's product overflows
-      if (zk > 0.f) share += zk * exp2f(mk - m) / z;
+      // zk 2^(mk - m) <= z, so neither factor's product overflows; a query head
+      // without a positive sum (NaN or +inf logits, or all -inf) leaves its KV
+      // head no coverage, kept key or not, as the group-mass form has it
+      share += z > 0.f ? zk * exp2f(mk - m) / z : NAN;
     }
   }
   red[jj][li] = share;
@@ -162,7 +164,7 @@ __global__ void __launch_bounds__(256) ratio_kernel(const __grid_constant__ Prob
     float s = 0.f;
 #pragma unroll
     for (int k = 0; k < 8; ++k) s += red[k][li];
-    cov[(((size_t)l * P.B + b) * P.Hkv + h) * P.Np + i] = s / (float)P.r;
+    cov[(((size_t)l * P.B + b) * P.Hkv + h) * P.Np + i] = s >= 0.f ? s / (float)P.r : 0.f;
   }
 }
 

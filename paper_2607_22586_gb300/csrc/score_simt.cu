@@ -156,7 +156,10 @@ __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <typename T, int D>
+// RATIO: the sums feed a ratio (coverage), over at most bf.kept_len keys where
+// given; a NaN logit then makes its row's sum NaN, also where all logits of its
+// 16 keys are NaN, which the selection's maxima pass over.
+template <typename T, int D, bool RATIO>
 __global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Problem P, Buffers bf,
                                                   const T* K, int nrank, bool vec) {
   dependent_start();
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Pro
   const int t_len = P.req[b].t_len, tok_off = P.req[b].tok_off;
   const int t0 = sl * P.split_len;
   int t1 = min(t_len, t0 + P.split_len);
-  if (bf.kept_len) t1 = min(t1, bf.kept_len[((size_t)l * P.B + b) * P.Hkv + h]);
+  if (RATIO && bf.kept_len) t1 = min(t1, bf.kept_len[((size_t)l * P.B + b) * P.Hkv + h]);
   const int tid = threadIdx.x, ty = tid / 16, tx = tid % 16;
   // this CTA's tiles of the split: rank r takes tiles [r, r + 1) * ntiles / nrank
   const int ntiles = max(0, t1 - t0 + TK - 1) / TK;
@@ -224,7 +227,7 @@ __global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Pro
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           x[j] = tk + half * TRUN + tx * 4 + j < t1 ? logit(acc, i, half * 4 + j) * P.alpha : -INFINITY;
-          m = fmaxf(m, x[j]);
+          m = fmaxf(m, RATIO && x[j] != x[j] ? INFINITY : x[j]);
         }
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
         m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
@@ -439,7 +442,7 @@ bool quad_loads(const Problem& P, const void* K) {
   return reinterpret_cast<uintptr_t>(K) % quad == 0 && (P.ls_kv * sizeof(T)) % quad == 0;
 }
 
-template <typename T, int D>
+template <typename T, int D, bool RATIO>
 cudaError_t launch_pass1(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K) {
   int nsm = 0;
   cudaError_t e = device_sms(&nsm);
@@ -458,9 +461,9 @@ cudaError_t launch_pass1(const Problem& P, const Buffers& bf, cudaStream_t st, c
   while (nrank < 8 && nrank < max_tiles && units * nrank < 3LL * nsm) nrank *= 2;
   const int runs = 2 * ((max_tiles + nrank - 1) / nrank);
   const size_t sm1 = (size_t)(TR * D + 2 * KC * TK) * sizeof(float) + (size_t)runs * TR * sizeof(float2);
-  if ((e = cudaFuncSetAttribute(pass1_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if ((e = cudaFuncSetAttribute(pass1_simt<T, D, RATIO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sm1)) != cudaSuccess) return e;
-  return launch_kernel(pass1_simt<T, D>, dim3((unsigned)(P.Hkv * P.total_splits * n_rt * nrank), P.L), TNT,
+  return launch_kernel(pass1_simt<T, D, RATIO>, dim3((unsigned)(P.Hkv * P.total_splits * n_rt * nrank), P.L), TNT,
                        sm1, st, P.overlap, nrank, P, bf, (const T*)K, nrank, vec);
 }
 
@@ -472,7 +475,7 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
   if (e != cudaSuccess) return e;
   const bool vec = quad_loads<T>(P, K);
   if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
-  if ((e = launch_pass1<T, D>(P, bf, st, K)) != cudaSuccess) return e;
+  if ((e = launch_pass1<T, D, false>(P, bf, st, K)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   if ((e = launch_merge(P, bf, st)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
@@ -536,9 +539,10 @@ cudaError_t launch_merge(const Problem& P, const Buffers& bf, cudaStream_t st) {
 cudaError_t launch_softmax_simt(const Problem& P, const Buffers& bf, cudaStream_t st,
                                 const void* K) {
   if (P.dtype == MMSHIFT_BF16)
-    return P.d == 128 ? launch_pass1<__nv_bfloat16, 128>(P, bf, st, K)
-                      : launch_pass1<__nv_bfloat16, 64>(P, bf, st, K);
-  return P.d == 128 ? launch_pass1<float, 128>(P, bf, st, K) : launch_pass1<float, 64>(P, bf, st, K);
+    return P.d == 128 ? launch_pass1<__nv_bfloat16, 128, true>(P, bf, st, K)
+                      : launch_pass1<__nv_bfloat16, 64, true>(P, bf, st, K);
+  return P.d == 128 ? launch_pass1<float, 128, true>(P, bf, st, K)
+                    : launch_pass1<float, 64, true>(P, bf, st, K);
 }
 
 cudaError_t launch_score_simt(const Problem& P, const Buffers& bf, cudaStream_t st,

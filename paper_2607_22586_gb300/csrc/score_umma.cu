@@ -262,10 +262,17 @@ __device__ __forceinline__ void softmax_chunk(float (&v)[32], float alpha, float
 // The same with the reference always at the running max, so no exponent is
 // positive and the largest terms carry no rounding of a large difference: for
 // sums whose ratio is the result (coverage), where the rounding of the
-// selection's sums would not cancel. Costs the max of every chunk.
+// selection's sums would not cancel. Costs the max of every chunk. A NaN logit
+// makes z NaN, also where every other column so far is masked or -inf (the max
+// alone would pass over it).
 __device__ __forceinline__ void softmax_chunk_max(const float (&v)[32], float alpha, float& m, float& z) {
   const float mn = fmaxf(m, max32(v) * alpha);
-  if (mn == -INFINITY) return;     // every column masked so far
+  if (mn == -INFINITY) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j)
+      if (v[j] != v[j]) z = v[j];
+    return;
+  }
   z = fmaf(z, fast_exp2(m - mn), exp2_sum32(v, pk2(alpha, alpha), mn));
   m = mn;
 }
@@ -856,6 +863,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         }
       }
       if (!ok) break;
+      // a NaN sum keeps its place in every merge: no partial is above +inf
+      if (RATIO && z_run != z_run) m_run = INFINITY;
       *dst = make_float2(m_run, z_run);
     }
   }
