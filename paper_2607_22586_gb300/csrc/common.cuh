@@ -196,7 +196,10 @@ __device__ __forceinline__ void set_status(int* status, int bit) {
 // Start of every kernel that may be launched as a programmatic dependent: the
 // next kernel of the call may take its place on the SMs, and everything the
 // kernels before this one wrote is visible afterwards. Without the launch
-// attribute both are no-ops.
+// attribute both are no-ops. What those kernels wrote is read by plain loads: a
+// non-coherent one (__ldg) is for memory nobody writes during the kernel's life,
+// which now begins while the kernel before still runs, and the compiler may move
+// it above the wait. K, V and the window queries are inputs and may be read so.
 __device__ __forceinline__ void dependent_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");

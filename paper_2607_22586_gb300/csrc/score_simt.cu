@@ -40,14 +40,24 @@ __device__ __forceinline__ void find_split(const Problem& P, int s, int& b, int&
   sl = s - P.req[b].split_off;
 }
 
-// Four consecutive elements as float32 (`vec`: the pointer allows one load).
-__device__ __forceinline__ float4 load4(const float* p, bool vec) {
-  if (vec) return __ldg(reinterpret_cast<const float4*>(p));
-  return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+// A value the call's input keeps for the whole call (INPUT: by the non-coherent
+// path), or one an earlier kernel of the call wrote.
+template <bool INPUT, typename V>
+__device__ __forceinline__ V load(const V* p) {
+  if constexpr (INPUT) return __ldg(p);
+  else return *p;
 }
+
+// Four consecutive elements as float32 (`vec`: the pointer allows one load).
+template <bool INPUT>
+__device__ __forceinline__ float4 load4(const float* p, bool vec) {
+  if (vec) return load<INPUT>(reinterpret_cast<const float4*>(p));
+  return make_float4(load<INPUT>(p), load<INPUT>(p + 1), load<INPUT>(p + 2), load<INPUT>(p + 3));
+}
+template <bool INPUT>
 __device__ __forceinline__ float4 load4(const __nv_bfloat16* p, bool vec) {
   if (vec) {
-    const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+    const uint2 u = load<INPUT>(reinterpret_cast<const uint2*>(p));
     return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
                        __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
   }
@@ -61,10 +71,10 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p, bool vec) {
 template <int R>
 __device__ __forceinline__ int tile_at(int row, int k) { return k * R + (row ^ (((k >> 2) & 3) << 3)); }
 
-// R rows x KD dimensions of src (rows `stride` elements apart, zeros from row n
+// R rows x KD dimensions of src (INPUT as above; rows `stride` elements apart, zeros from row n
 // on), read into registers and stored to a tile in two steps, so that the
 // reads of the next piece are in flight during the FMAs of the current one.
-template <typename T, int R, int KD>
+template <typename T, int R, int KD, bool INPUT>
 struct Piece {
   static constexpr int NB = (R / 8) * (KD / 16) / (TNT / 32);   // 8-row x 16-dimension blocks per warp
   float4 v[NB];
@@ -78,7 +88,7 @@ struct Piece {
     for (int i = 0; i < NB; ++i) {
       int row, k;
       at(i, row, k);
-      v[i] = row < n ? load4(src + (size_t)row * stride + k, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[i] = row < n ? load4<INPUT>(src + (size_t)row * stride + k, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   }
   __device__ __forceinline__ void store(float* dst) const {
@@ -191,7 +201,7 @@ __global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Pro
   // pieces of KC dimensions of the CTA's tiles, one after the other
   constexpr int NP = D / KC;
   const int np = (k1 - k0) * NP;
-  Piece<T, TK, KC> next;
+  Piece<T, TK, KC, true> next;
   auto fetch = [&](int p) {
     const int tk = t0 + (k0 + p / NP) * TK;
     next.load(kb + (size_t)tk * kstride + (p % NP) * KC, kstride, t1 - tk, vec);
@@ -200,7 +210,7 @@ __global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Pro
     fetch(0);
 #pragma unroll 1
     for (int c = 0; c < NP; ++c) {              // Prows_pad is a multiple of TR
-      Piece<T, TR, KC> a;
+      Piece<T, TR, KC, false> a;
       a.load(pk + c * KC, D, TR, true);
       a.store(As + c * KC * TR);
     }
@@ -368,7 +378,7 @@ __global__ void __launch_bounds__(TNT, 2) pass2_simt(const __grid_constant__ Pro
   // pieces of KC dimensions of the 64-row tiles, one after the other
   constexpr int NP = D / KC, CPT = TR / kChunk;
   const int np = (c_hi - c_lo + CPT - 1) / CPT * NP;
-  Piece<T, TR, KC> next;
+  Piece<T, TR, KC, false> next;
   auto fetch = [&](int p) {
     const int row0 = (c_lo + p / NP * CPT) * kChunk;
     next.load(pk + (size_t)row0 * D + (p % NP) * KC, D, P.Prows_pad - row0, true);
@@ -376,7 +386,7 @@ __global__ void __launch_bounds__(TNT, 2) pass2_simt(const __grid_constant__ Pro
   fetch(0);
 #pragma unroll 1
   for (int c = 0; c < NP; ++c) {
-    Piece<T, TK, KC> k;
+    Piece<T, TK, KC, true> k;
     k.load(kb + c * KC, kstride, t_len - kt, vec);
     k.store(Bs + c * KC * TK);
   }
@@ -392,7 +402,7 @@ __global__ void __launch_bounds__(TNT, 2) pass2_simt(const __grid_constant__ Pro
       clear(acc);
       const int row = c0 * kChunk + ty * 8;     // rows in eights: all or none inside
 #pragma unroll
-      for (int i = 0; i < 8; ++i) cn[i] = row < P.Prows_pad ? __ldg(cv + row + i) : INFINITY;
+      for (int i = 0; i < 8; ++i) cn[i] = row < P.Prows_pad ? cv[row + i] : INFINITY;
     }
     tile_dot(As + (p & 1) * KC * TR, Bs + pc * KC * TK, ty, tx, acc);
     if (p + 1 < np) next.store(As + ((p + 1) & 1) * KC * TR);

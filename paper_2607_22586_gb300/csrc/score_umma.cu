@@ -956,7 +956,7 @@ __global__ void __launch_bounds__(ANT) anchor_final_kernel(const __grid_constant
 #pragma unroll
       for (int j = 0; j < kMaxSplitAnchor; ++j) {
         const int t = t1st + i * ANT;
-        y[i][j] = t < t1 && j < P.r ? __ldg(y0 + (size_t)j * P.total_T + t) : 0.f;
+        y[i][j] = t < t1 && j < P.r ? y0[(size_t)j * P.total_T + t] : 0.f;
       }
   };
   float y[KPT][kMaxSplitAnchor];
@@ -1021,7 +1021,7 @@ __global__ void __launch_bounds__(ANT) anchor_kernel(const __grid_constant__ Pro
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int t = t0 + (q * U + u) * 32 + lane;
-        v[q][u] = t < t_len ? __ldg(y + t) : -INFINITY;
+        v[q][u] = t < t_len ? y[t] : -INFINITY;
       }
     float m = -INFINITY, z = 0.f;
 #pragma unroll

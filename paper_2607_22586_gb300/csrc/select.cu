@@ -76,7 +76,7 @@ struct SmemKeys {
 struct GlobalFloats {
   static constexpr bool kGlobal = true;
   const float* gmem;
-  __device__ __forceinline__ uint32_t operator()(int i) const { return nonneg_key(__ldg(gmem + i)); }
+  __device__ __forceinline__ uint32_t operator()(int i) const { return nonneg_key(gmem[i]); }
 };
 
 // Weight of a key (of a non-negative float x) in 2^-shift units: x * 2^shift
@@ -246,7 +246,7 @@ __device__ __forceinline__ void digit_histogram(const Src& get, int n, uint32_t 
 #pragma unroll
       for (int j = 0; j < U4; ++j) {
         const int i4 = base + j * NTH + tid;
-        f[j] = i4 < n4 ? __ldg(g4 + i4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        f[j] = i4 < n4 ? g4[i4] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
 #pragma unroll
       for (int j = 0; j < U4; ++j) {
@@ -440,7 +440,7 @@ __device__ int compact_prefix(const Src& get, int n, uint32_t prefix, int hs, ui
 #pragma unroll
       for (int j = 0; j < U4; ++j) {
         const int i4 = base + j * NTH + tid;
-        f[j] = i4 < n4 ? __ldg(g4 + i4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        f[j] = i4 < n4 ? g4[i4] : make_float4(0.f, 0.f, 0.f, 0.f);
       }
       uint32_t kk[4 * U4];
       bool va[4 * U4];
@@ -552,7 +552,7 @@ __device__ void total_and_max(const float* m, int n, int shift, uint32_t kspec, 
     if (k >= kspec) append(k, i);
   };
   const int head = min(n, (int)(((16u - (uint32_t)(reinterpret_cast<uintptr_t>(m) & 15)) & 15u) >> 2));
-  if (tid < head) add1(__ldg(m + tid), tid);
+  if (tid < head) add1(m[tid], tid);
   const float4* g4 = reinterpret_cast<const float4*>(m + head);
   const int n4 = (n - head) >> 2;
 #pragma unroll
@@ -595,7 +595,7 @@ __device__ void total_and_max(const float* m, int n, int shift, uint32_t kspec, 
   }
   carry();
   cp_async_wait<0>();
-  for (int i = head + (n4 << 2) + tid; i < n; i += NTH) add1(__ldg(m + i), i);
+  for (int i = head + (n4 << 2) + tid; i < n; i += NTH) add1(m[i], i);
   for (int off = 16; off; off >>= 1) {
     tot += __shfl_xor_sync(0xffffffffu, tot, off);
     km = max(km, __shfl_xor_sync(0xffffffffu, km, off));
@@ -646,7 +646,7 @@ __device__ int compact_above(const float* m, int n, uint32_t klb, uint32_t* cand
 #pragma unroll
     for (int j = 0; j < U4; ++j) {
       const int i4 = base + j * NTH + tid;
-      f[j] = i4 < n4 ? __ldg(g4 + i4) : make_float4(0.f, 0.f, 0.f, 0.f);
+      f[j] = i4 < n4 ? g4[i4] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     uint32_t kk[4 * U4];
     unsigned bal[4 * U4];
@@ -681,13 +681,13 @@ __device__ int compact_above(const float* m, int n, uint32_t klb, uint32_t* cand
     const int tail0 = head + (n4 << 2);
     const int i = tid < head ? tid : tail0 + (tid - 3);
     const bool has = tid < head || (tid >= 3 && tid < 6 && i < n);
-    const bool in = has && nonneg_key(__ldg(m + i)) >= klb;
+    const bool in = has && nonneg_key(m[i]) >= klb;
     const unsigned bl = __ballot_sync(0xffffffffu, in);
     if (bl) {
       unsigned at = 0;
       if (lane == 0) at = atomicAdd(&S.ncand, __popc(bl));
       at = __shfl_sync(0xffffffffu, at, 0) + __popc(bl & below);
-      if (in && at < (unsigned)cap) { cand[at] = nonneg_key(__ldg(m + i)); cidx[at] = (uint32_t)i; }
+      if (in && at < (unsigned)cap) { cand[at] = nonneg_key(m[i]); cidx[at] = (uint32_t)i; }
     }
   }
   __syncthreads();
@@ -1270,7 +1270,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(const __gr
 #pragma unroll
         for (int u = 0; u < UB4; ++u) {
           const int j4 = b4 + u * NT + lane;
-          a[u] = j4 < n4 ? __ldg(an4 + j4) : make_float4(0.f, 0.f, 0.f, 0.f);
+          a[u] = j4 < n4 ? an4[j4] : make_float4(0.f, 0.f, 0.f, 0.f);
           vt[u] = 0;
         }
         for (int g = 0; g < P.G; ++g) {
@@ -1278,7 +1278,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(const __gr
           for (int u = 0; u < UB4; ++u) {
             const int j4 = b4 + u * NT + lane;
             const uint32_t word =
-                j4 < n4 ? __ldg(bw + (size_t)g * P.total_words + (j4 >> 3)) : 0u;
+                j4 < n4 ? bw[(size_t)g * P.total_words + (j4 >> 3)] : 0u;
             const uint32_t nib = (word >> ((j4 & 7) * 4)) & 0xFu;
             // spread the nibble's bits into the bytes of vt
             vt[u] += (nib & 1u) | ((nib & 2u) << 7) | ((nib & 4u) << 14) | ((nib & 8u) << 21);
@@ -1320,7 +1320,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(const __gr
         for (int u = 0; u < UB; ++u) {
           vote[u] = 0;
           const int i = base0 + u * NT + lane;
-          av[u] = i < n ? __ldg(an + i) : 0.f;
+          av[u] = i < n ? an[i] : 0.f;
         }
         if (P.G <= 8) {
           // few groups: every lane reads the chunk's word of each group (one
@@ -1330,7 +1330,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(const __gr
 #pragma unroll
             for (int u = 0; u < UB; ++u) {
               const int base = base0 + u * NT;
-              word[u] = base < n ? __ldg(bw + (size_t)g * P.total_words + (base >> 5)) : 0u;
+              word[u] = base < n ? bw[(size_t)g * P.total_words + (base >> 5)] : 0u;
             }
 #pragma unroll
             for (int u = 0; u < UB; ++u) vote[u] += (word[u] >> lane) & 1u;
@@ -1351,7 +1351,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(const __gr
               const int g = (e * NT + tid) / NWD, wd = (e * NT + tid) % NWD;
               cand[wd * 32 + (g ^ (wd & 31))] =
                   g0 + g < P.G && b0 + 32 * wd < n
-                      ? __ldg(bw + (size_t)(g0 + g) * P.total_words + (b0 >> 5) + wd) : 0u;
+                      ? bw[(size_t)(g0 + g) * P.total_words + (b0 >> 5) + wd] : 0u;
             }
             __syncthreads();
 #pragma unroll
@@ -1375,7 +1375,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) topk_kernel(const __gr
 #pragma unroll
           for (int u = 0; u < UB; ++u) {
             const int i = base0 + u * NT + lane;
-            if (i < n) sv[u] += __ldg(gm + i);
+            if (i < n) sv[u] += gm[i];
           }
         }
       }
