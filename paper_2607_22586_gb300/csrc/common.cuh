@@ -284,9 +284,10 @@ cudaError_t launch_kept_rows(const Problem& P, const void* K, const int32_t* idx
                              int32_t* kept_len, int* status, cudaStream_t st);
 // cov = mean over the query heads of (sum over the kept keys) / (sum over all
 // keys) of each decode query's exponentials, from the two softmax passes'
-// partials: `all` over the prompt (problem P), `kept` over the kept rows (Pk).
-cudaError_t launch_coverage_ratio(const Problem& P, const Problem& Pk, const float2* all,
-                                  const float2* kept, float* cov, cudaStream_t st);
+// partials: `all` over the prompt (problem P), `kept` over the kept rows (Pk);
+// both may be overwritten.
+cudaError_t launch_coverage_ratio(const Problem& P, const Problem& Pk, float2* all, float2* kept,
+                                  float* cov, cudaStream_t st);
 // Attention-mass coverage of the kept set idx from the group masses in bf.
 cudaError_t launch_coverage(const Problem& P, const Buffers& bf, const int32_t* idx, float* cov,
                             cudaStream_t st);

@@ -122,36 +122,64 @@ __global__ void __launch_bounds__(KRT) kept_rows_kernel(const __grid_constant__ 
   }
 }
 
+// (m, z) += the partials src[0], src[step], ..., n of them, in order, eight loads
+// issued ahead.
+__device__ __forceinline__ void merge_run(const float2* src, size_t step, int n, float& m, float& z) {
+  constexpr int A = 8;
+  for (int s0 = 0; s0 < n; s0 += A) {
+    float2 v[A];
+#pragma unroll
+    for (int u = 0; u < A; ++u)
+      v[u] = s0 + u < n ? src[(size_t)(s0 + u) * step] : make_float2(-INFINITY, 0.f);
+#pragma unroll
+    for (int u = 0; u < A; ++u) merge_ms(m, z, v[u].x, v[u].y);
+  }
+}
+
+// Runs of kRun partials of every row merged into the run's first, a thread per
+// (row, run), where a row has more than one run: as one thread's chain a prompt's
+// partials (one per 256 keys) took longer than its softmax pass. 32 decode queries
+// of 28 / 4 heads, one layer, half the prompt kept: 128K keys 383 -> 148 us, 1M keys
+// 4,315 -> 1,491 (the group-mass form took 2,813); 28 layers of 32K keys, 2,048
+// kept rows, 128 partials a row: 327 -> 278.
+constexpr int kRun = 64;
+
+__global__ void __launch_bounds__(128) ratio_runs_kernel(const __grid_constant__ Problem Q, float2* part) {
+  const int row = (blockIdx.x % (Q.Prows_pad / 128)) * 128 + threadIdx.x;
+  const int s0 = blockIdx.x / (Q.Prows_pad / 128) * kRun, h = blockIdx.y;
+  const int l = blockIdx.z / Q.B, b = blockIdx.z % Q.B;
+  const int n = min(kRun, Q.req[b].nsplit * Q.part_slots - s0);
+  if (n <= 0 || row >= Q.Prows) return;
+  float2* src = part + ((((size_t)l * Q.Hkv + h) * Q.total_splits + Q.req[b].split_off) * Q.part_slots + s0) *
+                           Q.Prows_pad + row;
+  float m = -INFINITY, z = 0.f;
+  merge_run(src, Q.Prows_pad, n, m, z);
+  *src = make_float2(m, z);
+}
+
 // CTA = 32 decode queries of one (layer, request, KV head): thread (i, jj) merges
-// the partials of query i under query heads jj, jj + 8, ...
+// the partials of query i under query heads jj, jj + 8, ...; run, run_k: partials
+// already merged into each place that holds one.
 __global__ void __launch_bounds__(256) ratio_kernel(const __grid_constant__ Problem P,
                                                     const __grid_constant__ Problem Pk,
                                                     const float2* all, const float2* kept,
-                                                    float* cov) {
+                                                    int run, int run_k, float* cov) {
   __shared__ float red[8][33];
   const int li = threadIdx.x % 32, jj = threadIdx.x / 32;
   const int i = blockIdx.x * 32 + li, h = blockIdx.y;
   const int l = blockIdx.z / P.B, b = blockIdx.z % P.B;
   float share = 0.f;
   if (i < P.Np) {
-    auto merged = [&](const Problem& Q, const float2* part, int row, float& m, float& z) {
+    auto merged = [&](const Problem& Q, const float2* part, int step, int row, float& m, float& z) {
       const float2* src = part + (((size_t)l * Q.Hkv + h) * Q.total_splits + Q.req[b].split_off) *
                                      Q.part_slots * Q.Prows_pad + row;
       const int ns = Q.req[b].nsplit * Q.part_slots;
-      constexpr int A = 8;
-      for (int s0 = 0; s0 < ns; s0 += A) {
-        float2 v[A];
-#pragma unroll
-        for (int u = 0; u < A; ++u)
-          v[u] = s0 + u < ns ? src[(size_t)(s0 + u) * Q.Prows_pad] : make_float2(-INFINITY, 0.f);
-#pragma unroll
-        for (int u = 0; u < A; ++u) merge_ms(m, z, v[u].x, v[u].y);
-      }
+      merge_run(src, (size_t)step * Q.Prows_pad, (ns + step - 1) / step, m, z);
     };
     for (int j = jj; j < P.r; j += 8) {
       float m = -INFINITY, z = 0.f, mk = -INFINITY, zk = 0.f;
-      merged(P, all, j * P.gs + i, m, z);
-      merged(Pk, kept, j * P.gs + i, mk, zk);
+      merged(P, all, run, j * P.gs + i, m, z);
+      merged(Pk, kept, run_k, j * P.gs + i, mk, zk);
       // zk 2^(mk - m) <= z, so neither factor's product overflows; a query head
       // without a positive sum (NaN or +inf logits, or all -inf) leaves its KV
       // head no coverage, kept key or not, as the group-mass form has it
@@ -188,9 +216,22 @@ cudaError_t launch_kept_rows(const Problem& P, const void* K, const int32_t* idx
   return cudaGetLastError();
 }
 
-cudaError_t launch_coverage_ratio(const Problem& P, const Problem& Pk, const float2* all,
-                                  const float2* kept, float* cov, cudaStream_t st) {
-  ratio_kernel<<<dim3((P.Np + 31) / 32, P.Hkv, P.L * P.B), 256, 0, st>>>(P, Pk, all, kept, cov);
+cudaError_t launch_coverage_ratio(const Problem& P, const Problem& Pk, float2* all, float2* kept,
+                                  float* cov, cudaStream_t st) {
+  int run[2] = {1, 1};
+  for (int k = 0; k < 2; ++k) {
+    const Problem& Q = k ? Pk : P;
+    int ns = 0;
+    for (int b = 0; b < Q.B; ++b) ns = max(ns, Q.req[b].nsplit * Q.part_slots);
+    if (ns <= kRun) continue;
+    run[k] = kRun;
+    ratio_runs_kernel<<<dim3(Q.Prows_pad / 128 * ((ns + kRun - 1) / kRun), Q.Hkv, Q.L * Q.B), 128, 0, st>>>(
+        Q, k ? kept : all);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  ratio_kernel<<<dim3((P.Np + 31) / 32, P.Hkv, P.L * P.B), 256, 0, st>>>(P, Pk, all, kept, run[0], run[1],
+                                                                        cov);
   return cudaGetLastError();
 }
 
