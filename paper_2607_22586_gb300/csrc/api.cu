@@ -738,7 +738,10 @@ static mmshift_status run_coverage(CoverageJob& J, const void* K, const void* de
   bk.kept_len = klen;
   void* kept = ws + J.kept;
   cudaError_t e = launch_proxy_pack(P, bf, st, nullptr);
-  if (e == cudaSuccess) e = launch_kept_rows(P, K, idx, kept, klen, bf.status, st);
+  // its scratch is the prompt's softmax partials, at least 8 KB for each request and
+  // each 1024 keys of a (layer, KV head), which the pass after it writes
+  if (e == cudaSuccess)
+    e = launch_kept_rows(P, K, idx, kept, klen, reinterpret_cast<int32_t*>(bf.part), bf.status, st);
   if (e == cudaSuccess) e = P.use_umma ? launch_softmax_umma(P, bf, st, K) : launch_softmax_simt(P, bf, st, K);
   if (e == cudaSuccess) e = Q.use_umma ? launch_softmax_umma(Q, bk, st, kept) : launch_softmax_simt(Q, bk, st, kept);
   if (e == cudaSuccess) e = launch_coverage_ratio(P, Q, bf.part, bk.part, cov, st);

@@ -279,9 +279,10 @@ cudaError_t launch_anchor_split(const Problem& P, const Buffers& bf, cudaStream_
 cudaError_t launch_merge(const Problem& P, const Buffers& bf, cudaStream_t st);
 // Copies the kept rows of K (idx; -1 and bad indices left out, the bad ones
 // reported) to kept [L][R][Hkv][d], each (layer, request, KV head)'s rows
-// together from its first output row on, and their number to kept_len.
+// together from its first output row on, and their number to kept_len. scratch:
+// at least L * Hkv * (R / 256 + B) words, free again afterwards.
 cudaError_t launch_kept_rows(const Problem& P, const void* K, const int32_t* idx, void* kept,
-                             int32_t* kept_len, int* status, cudaStream_t st);
+                             int32_t* kept_len, int32_t* scratch, int* status, cudaStream_t st);
 // cov = mean over the query heads of (sum over the kept keys) / (sum over all
 // keys) of each decode query's exponentials, from the two softmax passes'
 // partials: `all` over the prompt (problem P), `kept` over the kept rows (Pk);

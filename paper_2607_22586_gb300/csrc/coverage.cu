@@ -66,16 +66,36 @@ __global__ void __launch_bounds__(kCovThreads) coverage_kernel(Problem P, const 
     cov[(((size_t)l * P.B + b) * P.Hkv + h) * P.G + g] = tot > 0.f ? kept / tot : 0.f;
 }
 
-// CTA = 256 consecutive kept-set entries of one (layer, request, KV head). The
-// entries before them are counted again by every CTA (at most the budget, a
-// strided read from L2), which spares a separate scan.
+// CTA = 256 consecutive kept-set entries (a chunk) of one (layer, request, KV
+// head). The valid entries before them, which say where its rows go, come from
+// the chunks' counts (kept_count_kernel) or, up to kCountAgain entries, are counted
+// again by every CTA, which spares a launch of 2 to 4 us but grows with the square
+// of the budget. One layer of 128K keys, 28 / 4 heads, counts against counting
+// again: 8,192 kept rows 98 and 94 us a call, 16,384 104 and 102, 65,536 133 and 148.
 constexpr int KRT = 256;
+constexpr int kCountAgain = 16384;
+
+// Chunk counts [L][Hkv][R / KRT + B], request b's from R.out_off / KRT + b on.
+__device__ __forceinline__ size_t chunk_at(const Problem& P, int l, int h, int b) {
+  return ((size_t)l * P.Hkv + h) * (P.R / KRT + P.B) + P.req[b].out_off / KRT + b;
+}
+
+__global__ void __launch_bounds__(KRT) kept_count_kernel(const __grid_constant__ Problem P,
+                                                         const int32_t* idx, int32_t* counts) {
+  const int h = blockIdx.y, l = blockIdx.z / P.B, b = blockIdx.z % P.B;
+  const ReqInfo R = P.req[b];
+  const int c = blockIdx.x * KRT + threadIdx.x;
+  if (blockIdx.x * KRT >= R.keep) return;
+  const int t = c < R.keep ? idx[((size_t)l * P.R + R.out_off + c) * P.Hkv + h] : -1;
+  const int n = __syncthreads_count((unsigned)t < (unsigned)R.t_len);
+  if (threadIdx.x == 0) counts[chunk_at(P, l, h, b) + blockIdx.x] = n;
+}
 
 template <int ROWB>
 __global__ void __launch_bounds__(KRT) kept_rows_kernel(const __grid_constant__ Problem P,
                                                         const uint8_t* K, const int32_t* idx,
-                                                        uint8_t* kept, int32_t* kept_len,
-                                                        int* status, bool vec) {
+                                                        const int32_t* counts, uint8_t* kept,
+                                                        int32_t* kept_len, int* status, bool vec) {
   constexpr int LPR = ROWB / 16;   // lanes per row
   const int h = blockIdx.y, l = blockIdx.z / P.B, b = blockIdx.z % P.B;
   const ReqInfo R = P.req[b];
@@ -84,7 +104,12 @@ __global__ void __launch_bounds__(KRT) kept_rows_kernel(const __grid_constant__ 
   const int32_t* id = idx + ((size_t)l * P.R + R.out_off) * P.Hkv + h;
   __shared__ int wsum[KRT / 32], wcnt[KRT / 32], list[KRT];
   int before = 0;
-  for (int c = tid; c < start; c += KRT) before += (unsigned)id[(size_t)c * P.Hkv] < (unsigned)R.t_len;
+  if (counts) {
+    const int32_t* cnt = counts + chunk_at(P, l, h, b);
+    for (int c = tid; c < (int)blockIdx.x; c += KRT) before += cnt[c];
+  } else {
+    for (int c = tid; c < start; c += KRT) before += (unsigned)id[(size_t)c * P.Hkv] < (unsigned)R.t_len;
+  }
   before = __reduce_add_sync(0xffffffffu, before);
   const int c = start + tid;
   const int t = c < R.keep ? id[(size_t)c * P.Hkv] : -1;
@@ -199,7 +224,7 @@ __global__ void __launch_bounds__(256) ratio_kernel(const __grid_constant__ Prob
 }  // namespace
 
 cudaError_t launch_kept_rows(const Problem& P, const void* K, const int32_t* idx, void* kept,
-                             int32_t* kept_len, int* status, cudaStream_t st) {
+                             int32_t* kept_len, int32_t* scratch, int* status, cudaStream_t st) {
   int maxk = 0;
   for (int b = 0; b < P.B; ++b) maxk = max(maxk, P.req[b].keep);
   const dim3 grid((maxk + KRT - 1) / KRT, P.Hkv, P.L * P.B);
@@ -207,10 +232,16 @@ cudaError_t launch_kept_rows(const Problem& P, const void* K, const int32_t* idx
   const bool vec = ((reinterpret_cast<uintptr_t>(K) | (uintptr_t)(P.ls_kv * esz)) & 15) == 0;
   const uint8_t* k = static_cast<const uint8_t*>(K);
   uint8_t* o = static_cast<uint8_t*>(kept);
+  int32_t* counts = maxk > kCountAgain ? scratch : nullptr;
+  if (counts) {
+    kept_count_kernel<<<grid, KRT, 0, st>>>(P, idx, counts);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   switch (P.d * esz) {
-    case 128: kept_rows_kernel<128><<<grid, KRT, 0, st>>>(P, k, idx, o, kept_len, status, vec); break;
-    case 256: kept_rows_kernel<256><<<grid, KRT, 0, st>>>(P, k, idx, o, kept_len, status, vec); break;
-    case 512: kept_rows_kernel<512><<<grid, KRT, 0, st>>>(P, k, idx, o, kept_len, status, vec); break;
+    case 128: kept_rows_kernel<128><<<grid, KRT, 0, st>>>(P, k, idx, counts, o, kept_len, status, vec); break;
+    case 256: kept_rows_kernel<256><<<grid, KRT, 0, st>>>(P, k, idx, counts, o, kept_len, status, vec); break;
+    case 512: kept_rows_kernel<512><<<grid, KRT, 0, st>>>(P, k, idx, counts, o, kept_len, status, vec); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

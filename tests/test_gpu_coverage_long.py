@@ -1,8 +1,9 @@
 """mmshift_coverage of long prompts. A row's softmax partials (four per 1,024 keys
 on the tensor cores, one on the CUDA cores) are merged in runs of 64 first where
 they exceed one run: just below and above one run, last runs of one partial, short
-requests beside long ones, in the prompt's sums and in the kept rows' as well.
-Reference and bounds as in the tests of the kept rows."""
+requests beside long ones, in the prompt's sums and in the kept rows' as well. The
+kept rows of budgets above 16,384 are placed by their chunks' counts: one more
+than that, several requests and layers, padding rows anywhere. Reference and bounds as in the tests of the kept rows."""
 import math
 
 import pytest
@@ -43,4 +44,14 @@ def _check(lens, budgets, hq, hkv, d, L, n_dec, dtype):
     ((66000,), (500,), 2, 1, 64, 1, 9, "f32"),                  # CUDA cores: 65 partials
 ])
 def test_coverage_of_long_prompts(lens, budgets, hq, hkv, d, L, n_dec, dtype):
+    _check(lens, budgets, hq, hkv, d, L, n_dec, dtype)
+
+
+@pytest.mark.parametrize("lens,budgets,hq,hkv,d,L,n_dec,dtype", [
+    ((40000,), (16384,), 8, 2, 128, 1, 40, "bf16"),             # counted again by each CTA
+    ((40000,), (16385,), 8, 2, 128, 1, 40, "bf16"),             # counts, a last chunk of one entry
+    ((300, 50000, 1, 700), (77, 17000, 1, 256), 14, 2, 128, 2, 33, "bf16"),
+    ((40000, 300), (16640, 257), 4, 1, 64, 1, 70, "f32"),
+])
+def test_coverage_of_large_budgets(lens, budgets, hq, hkv, d, L, n_dec, dtype):
     _check(lens, budgets, hq, hkv, d, L, n_dec, dtype)
