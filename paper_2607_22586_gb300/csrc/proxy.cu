@@ -435,16 +435,14 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
   }
 }
 
-// Every element of a call without a list, recomputed in float64: one thread per
-// element or rotated pair. All float64 units are busy, so the parts of an element
-// side by side (refine_kernel) would only wait for one another: 28 heads, N = 512,
-// rotated, 2,541 us with one thread per element, 2,574 us side by side, 1,294 us
-// with one thread per pair.
+// Every element of a call recomputed in float64, for one without a list or with
+// more entries than its list holds: one thread per element or rotated pair. All
+// float64 units are busy, so the parts of an element side by side (refine_kernel)
+// would only wait for one another: 28 heads, N = 512, proxy stage of an overflowing
+// call 895 us side by side, 674 us like this; rotated 1,642 and 889 us. A call of
+// its own: inlined in refine_kernel it cost few-proxy calls of 28 layers 3 to 5 us.
 template <int D>
-__global__ void __launch_bounds__(128) refine_all_kernel(const __grid_constant__ Problem P,
-                                                         const __grid_constant__ Buffers bf,
-                                                         const __nv_bfloat16* qwin) {
-  dependent_start();
+__device__ __noinline__ void refine_every(const Problem& P, const Buffers& bf, const __nv_bfloat16* qwin) {
   constexpr int half = D / 2;
   const bool rope = P.rope_theta > 0.f;
   const int64_t n = (int64_t)P.L * P.B * P.Hq * P.Np * (rope ? half : D);
@@ -469,6 +467,15 @@ __global__ void __launch_bounds__(128) refine_all_kernel(const __grid_constant__
   }
 }
 
+// A call without a list.
+template <int D>
+__global__ void __launch_bounds__(128) refine_all_kernel(const __grid_constant__ Problem P,
+                                                         const __grid_constant__ Buffers bf,
+                                                         const __nv_bfloat16* qwin) {
+  dependent_start();
+  refine_every<D>(P, bf, qwin);
+}
+
 // Elements the sampler found undecided, recomputed in float64: mu + (gamma
 // sigma) z from the same Philox words, rotated, rounded to bf16 into the packed
 // block and the caller-layout copy. A CTA takes 32 elements at a time, one warp
@@ -478,7 +485,7 @@ __global__ void __launch_bounds__(128) refine_all_kernel(const __grid_constant__
 // logarithm and sine, which the warps run side by side (against one thread per
 // element, proxy stage of one layer of 28 heads, N = 512: 30.1 -> 25.8 us, of the
 // 28-layer 32K stack with few proxies 42.0 -> 33.7 us). A call whose entries
-// overflowed the list has every element recomputed.
+// overflowed the list has every element recomputed (refine_every).
 template <int D>
 __global__ void __launch_bounds__(224) refine_kernel(const __grid_constant__ Problem P,
                                                      const __grid_constant__ Buffers bf,
@@ -489,29 +496,22 @@ __global__ void __launch_bounds__(224) refine_kernel(const __grid_constant__ Pro
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const bool rope = P.rope_theta > 0.f;
   const int cnt = *bf.refine_count;
-  const bool list = cnt <= bf.refine_cap;
-  const int64_t n = list ? cnt : (int64_t)P.L * P.B * P.Hq * P.Np * D;
-  for (int64_t base = (int64_t)blockIdx.x * 32; base < n; base += (int64_t)gridDim.x * 32) {
+  if (cnt > bf.refine_cap) {
+    refine_every<D>(P, bf, qwin);
+    return;
+  }
+  for (int64_t base = (int64_t)blockIdx.x * 32; base < cnt; base += (int64_t)gridDim.x * 32) {
     const int64_t e = base + lane;
     int l = 0, b = 0, hq = 0, i = 0, dd = 0;
-    if (e < n) {
-      if (list) {
-        const uint64_t it = bf.refine_wide ? reinterpret_cast<const uint64_t*>(bf.refine_items)[e]
-                                           : (uint64_t)bf.refine_items[e];
-        const int lb = (int)(it >> bf.refine_lb_bit);
-        l = lb / P.B;
-        b = lb - l * P.B;
-        hq = (int)((uint32_t)(it >> bf.refine_hq_bit) & ((1u << (bf.refine_lb_bit - bf.refine_hq_bit)) - 1u));
-        i = (int)((uint32_t)it & ((1u << bf.refine_hq_bit) - 1u)) / D;
-        dd = (int)((uint32_t)it % D);
-      } else {
-        int64_t r = e;
-        dd = (int)(r % D); r /= D;
-        i = (int)(r % P.Np); r /= P.Np;
-        hq = (int)(r % P.Hq); r /= P.Hq;
-        b = (int)(r % P.B);
-        l = (int)(r / P.B);
-      }
+    if (e < cnt) {
+      const uint64_t it = bf.refine_wide ? reinterpret_cast<const uint64_t*>(bf.refine_items)[e]
+                                         : (uint64_t)bf.refine_items[e];
+      const int lb = (int)(it >> bf.refine_lb_bit);
+      l = lb / P.B;
+      b = lb - l * P.B;
+      hq = (int)((uint32_t)(it >> bf.refine_hq_bit) & ((1u << (bf.refine_lb_bit - bf.refine_hq_bit)) - 1u));
+      i = (int)((uint32_t)it & ((1u << bf.refine_hq_bit) - 1u)) / D;
+      dd = (int)((uint32_t)it % D);
       const int f = dd % half;
       if (warp < 6) {
         const int c = warp / 3;                    // element of the pair
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(224) refine_kernel(const __grid_constant__ Pro
       }
     }
     __syncthreads();
-    if (warp == 0 && e < n) {
+    if (warp == 0 && e < cnt) {
       auto value = [&](int c) {
         const double z = __dmul_rn(rad[c][lane], trig[c][lane]);
         return __dadd_rn(mu[c][lane], __dmul_rn(__dmul_rn((double)P.gamma, sig[c][lane]), z));
