@@ -3,6 +3,7 @@ of one workload shape and calls ``mmshift_select`` on the current stream.
 PyTorch only provides device memory and streams here."""
 from __future__ import annotations
 
+from contextlib import nullcontext
 from typing import Optional, Sequence
 
 import torch
@@ -44,6 +45,22 @@ class KVSelector:
 
     def _stream(self, stream):
         return torch.cuda.current_stream(self.device) if stream is None else stream
+
+    def _buffers_of(self, stream):
+        """Context in which buffers belong to the call's stream: a workspace of
+        another stream could still be in use there, would be zeroed too late and
+        could be handed out again while the call runs."""
+        if stream is None:
+            return nullcontext()
+        if not isinstance(stream, torch.cuda.Stream):
+            stream = torch.cuda.ExternalStream(int(getattr(stream, "cuda_stream", stream)), device=self.device)
+        return torch.cuda.stream(stream)
+
+    def _results_of(self, stream, out):
+        """A result made on the call's stream, for use on the current one."""
+        if stream is not None:
+            out.record_stream(torch.cuda.current_stream(self.device))
+        return out
 
     def _check(self, *ts):
         for t in ts:
@@ -89,12 +106,13 @@ class KVSelector:
         [L, T_total, Hq, d] -> [L, B, 2, Hq*d] float32 (mean, std)."""
         self._check(qfull)
         n = L.mmshift_prefill_stats_workspace_size(self.shape)
-        ws = torch.empty(max(n, 1), dtype=torch.uint8, device=self.device)
-        out = torch.empty((self.n_layers, len(self.budgets), 2, self.n_q_heads * self.head_dim),
-                          dtype=torch.float32, device=self.device)
+        with self._buffers_of(stream):
+            ws = torch.empty(max(n, 1), dtype=torch.uint8, device=self.device)
+            out = torch.empty((self.n_layers, len(self.budgets), 2, self.n_q_heads * self.head_dim),
+                              dtype=torch.float32, device=self.device)
         L.check(L.mmshift_prefill_stats(self.shape, qfull, layer_stride, out, ws, n, self._stream(stream)),
                 "mmshift_prefill_stats")
-        return out
+        return self._results_of(stream, out)
 
     def coverage(self, K: torch.Tensor, qwin: torch.Tensor, dec_q: torch.Tensor,
                  idx: Optional[torch.Tensor] = None, softmax_scale: float = 0.0,
@@ -105,19 +123,20 @@ class KVSelector:
         self._check(K, qwin, dec_q)
         n_dec = dec_q.shape[3]
         n = L.mmshift_coverage_workspace_size(self.shape, n_dec)
-        # only the status word, in the first 256 bytes, has to start at zero
-        if n <= 1 << 23:
-            ws = torch.zeros(n, dtype=torch.uint8, device=self.device)
-        else:
-            ws = torch.empty(n, dtype=torch.uint8, device=self.device)
-            ws[:256].zero_()
-        out = torch.empty((self.n_layers, len(self.budgets), self.n_kv_heads, n_dec),
-                          dtype=torch.float32, device=self.device)
+        with self._buffers_of(stream):
+            # only the status word, in the first 256 bytes, has to start at zero
+            if n <= 1 << 23:
+                ws = torch.zeros(n, dtype=torch.uint8, device=self.device)
+            else:
+                ws = torch.empty(n, dtype=torch.uint8, device=self.device)
+                ws[:256].zero_()
+            out = torch.empty((self.n_layers, len(self.budgets), self.n_kv_heads, n_dec),
+                              dtype=torch.float32, device=self.device)
         L.check(L.mmshift_coverage(self.shape, K, qwin, dec_q, n_dec, softmax_scale,
                                    self.out_idx if idx is None else idx, out, ws, n,
                                    self._stream(stream)), "mmshift_coverage")
         L.check(L.mmshift_poll_status(ws, self._stream(stream)), "mmshift_coverage status")
-        return out
+        return self._results_of(stream, out)
 
     def poll(self, stream=None) -> None:
         if stream is None:
