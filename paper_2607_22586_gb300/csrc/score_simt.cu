@@ -21,9 +21,9 @@
 //   a time in ascending order, into the group masses and the anchor (mean over
 //   the r anchor rows).
 #include <algorithm>
-#include <cmath>
 
 #include "common.cuh"
+#include "group_ranges.h"
 #include "umma.cuh"
 
 namespace mmshift {
@@ -334,18 +334,18 @@ __global__ void merge_kernel(const __grid_constant__ Problem P, const __grid_con
 
 template <typename T, int D>
 __global__ void __launch_bounds__(TNT, 2) pass2_simt(const __grid_constant__ Problem P, Buffers bf,
-                                                  const T* K, int gper, int ngr, bool own, bool vec) {
+                                                  const T* K, GroupRanges gr, bool vec) {
   dependent_start();
   extern __shared__ float sm[];
   float* Bs = sm;                    // [D][128] keys (stationary)
   float* As = Bs + TK * D;           // [2][KC][64] proxy rows, a piece and the next one
   float* sums = As + 2 * KC * TR;    // [4][128] sums over 16 rows
-  // ranges of gper groups; the anchor (group G) is a last range of its own, or
-  // part of the last one. The longest start first.
-  const int l = blockIdx.y, per = gridDim.x / ngr;
-  const int range = own ? (int)blockIdx.x / per : ngr - 1 - (int)blockIdx.x / per;
+  // the longest ranges start first
+  const int l = blockIdx.y, per = gridDim.x / gr.ngr;
+  const int range = gr.own ? (int)blockIdx.x / per : gr.ngr - 1 - (int)blockIdx.x / per;
   int u = blockIdx.x % per;
-  const int g0 = min(P.G, range * gper), g1 = range == ngr - 1 ? P.G + 1 : min(P.G, g0 + gper);
+  int g0, g1;
+  range_groups(gr, P.G, range, g0, g1);
   const int h = u % P.Hkv;
   u /= P.Hkv;
   int b = 0;
@@ -489,44 +489,15 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   if ((e = launch_merge(P, bf, st)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
-  // pass 2: the groups in ranges spread over CTAs. An SM takes n CTAs two at a time
-  // and a last odd one alone at about 0.6 of the rate, each for its 64-row tiles
-  // and about half a tile more for its keys; the anchor goes with the last
-  // range (about 0.3 of a tile for its sums) or alone, beside an odd CTA if there
-  // is one. Of all range lengths the one with the least time by that. Ranges for
-  // about three rounds of two CTAs, the anchor counted as a group, left last
-  // rounds nearly empty and tiles partly filled: 4001 keys, 8 groups of 112 rows,
-  // 263 us a call in ranges of two groups, 242 of four; 346 keys over eight KV heads
-  // 126 -> 97; 42 calls of 200 to 4000 keys 3 % less on average.
   long long tiles = 0;
   for (int b = 0; b < P.B; ++b) tiles += (P.req[b].t_len + TK - 1) / TK;
   const long long keyu = tiles * P.Hkv * P.L;
-  const int G1 = std::max(P.G, 1);
-  int gper = G1, ngr = 1;
-  bool own = false;
-  double best = -1;
-  for (int n = 1; n <= G1; ++n) {
-    const int len = (G1 + n - 1) / n;              // groups per range
-    if ((G1 + len - 1) / len != n) continue;       // the same length as a smaller n
-    const double ctas = (double)((keyu * n + nsm - 1) / nsm), odd = ctas - 2 * std::floor(ctas / 2);
-    for (int alone = 0; alone <= (P.G ? 1 : 0); ++alone) {
-      const int last = (P.G - (n - 1) * len) * P.RG + (alone ? 0 : P.anchor_rows);
-      const double each = std::max((std::min(len, P.G) * P.RG + TR - 1) / TR + 0.5,
-                                   (last + TR - 1) / TR + (alone ? 0.5 : 0.8));
-      const double time = ctas * each + std::max(0.67 * odd * each, alone ? 1.5 * keyu / nsm : 0.0);
-      if (best < 0 || time < best) {
-        best = time;
-        gper = len;
-        own = alone != 0;
-        ngr = n + alone;
-      }
-    }
-  }
+  const GroupRanges gr = choose_ranges(P.G, P.RG, P.anchor_rows, TR, keyu, nsm);
   const size_t sm2 = (size_t)(TK * D + 2 * KC * TR + 4 * TK) * sizeof(float);
   if ((e = cudaFuncSetAttribute(pass2_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)sm2)) != cudaSuccess) return e;
-  return launch_kernel(pass2_simt<T, D>, dim3((unsigned)(tiles * P.Hkv * ngr), P.L), TNT, sm2, st,
-                       P.overlap, 0, P, bf, (const T*)K, gper, ngr, own, vec);
+  return launch_kernel(pass2_simt<T, D>, dim3((unsigned)(tiles * P.Hkv * gr.ngr), P.L), TNT, sm2, st,
+                       P.overlap, 0, P, bf, (const T*)K, gr, vec);
 }
 
 }  // namespace
