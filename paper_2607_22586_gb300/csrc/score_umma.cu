@@ -306,15 +306,15 @@ __device__ __forceinline__ void mass_chunk(const float (&v)[16], const uint64_t 
   }
 }
 
-// Sum over the ncols (multiple of 8) accumulator columns of one group:
+// Sum over the ncols (multiple of 8) accumulator columns of the anchor rows:
 // sum_j exp2(acc_j * alpha - c_j), column j feeding partial sum j mod 4 in
 // ascending order (the odd 16 columns first, so that the last load is a wide
 // one), the four partial sums added in a fixed order. nc points at the warp's
 // shared-memory copy of the block's negated normalisers; loaded() runs once,
 // when the last columns are in registers and before their exponentials.
 template <class Loaded>
-__device__ __forceinline__ float group_sum(uint32_t tcol, uint32_t nc, int ncols, float alpha,
-                                           const Loaded& loaded) {
+__device__ __forceinline__ float anchor_sum(uint32_t tcol, uint32_t nc, int ncols, float alpha,
+                                            const Loaded& loaded) {
   const uint64_t al2 = pk2(alpha, alpha);
   uint64_t a01 = 0, a23 = 0;       // (+0, +0)
   int cc = 0;
@@ -364,32 +364,34 @@ __device__ __forceinline__ float group_sum(uint32_t tcol, uint32_t nc, int ncols
   return (a0 + a1) + (a2 + a3);
 }
 
-// The same over NC chunks of 16 columns, unrolled: the tensor-memory load and
-// the normalisers of the next chunk are in flight during the exponentials of
-// the current one. With two draining warps per scheduler the loads of the loop
-// above are exposed: a 112-column sum takes 2,140 clocks there and 1,780 here
-// (448 is the MUFU time of its exponentials), the pass over the 28-layer 32K
-// stack 2.66 and 2.48 ms. Unrolled for the widths of 16 proxies per group under
-// GQA ratios 7 and 8; narrower groups have little to overlap.
+// The same over the columns of a group, NC chunks of 16, unrolled: the tensor-memory
+// load of the next chunk is in flight during the exponentials of the current one.
+// With two draining warps per scheduler the loads of the loop above are exposed: a
+// 112-column sum takes 2,140 clocks there and 1,780 so (448 is the MUFU time of
+// its exponentials).
+//
+// Every width has a kernel of its own: a choice by width inside one kernel costs
+// the widths that do not take it. Eight layers of 32K keys, d = 128, 32 groups, the
+// pass in us with two unrolled widths (112, 128) beside the loop, with the loop
+// alone, and like this: 16 columns 251, 220, 190; 64 columns 476, 454, 413; 96
+// columns 691, 676, 622; 128 columns 743, 793, 733; 16 groups of 256 columns 947,
+// 924, 780. (The normalisers of the next chunk loaded ahead as well: 2 to 5 % less
+// for most widths, but 72B-class short requests, two groups of 128, 448 -> 455.)
 template <int NC, class Loaded>
-__device__ __forceinline__ float group_sum_pipe(uint32_t tcol, uint32_t nc, float alpha,
-                                                const Loaded& loaded) {
+__device__ __forceinline__ float group_sum(uint32_t tcol, uint32_t nc, float alpha,
+                                           const Loaded& loaded) {
   const uint64_t al2 = pk2(alpha, alpha);
   uint64_t a01 = 0, a23 = 0;       // (+0, +0)
   float v[2][16];
-  uint64_t ncv[2][8];
+  uint64_t ncv[8];
   tmem_ld16(tcol, v[0]);
-  load_nc16(nc, ncv[0]);
 #pragma unroll
   for (int i = 0; i < NC; ++i) {
+    load_nc16(nc + 64 * i, ncv);
     tmem_wait_ld16(v[i & 1]);
-    if (i + 1 < NC) {
-      tmem_ld16(tcol + 16 * (i + 1), v[(i + 1) & 1]);
-      load_nc16(nc + 64 * (i + 1), ncv[(i + 1) & 1]);
-    } else {
-      loaded();
-    }
-    mass_chunk(v[i & 1], ncv[i & 1], al2, a01, a23);
+    if (i + 1 < NC) tmem_ld16(tcol + 16 * (i + 1), v[(i + 1) & 1]);
+    else loaded();
+    mass_chunk(v[i & 1], ncv, al2, a01, a23);
   }
   float a0, a1, a2, a3;
   upk2(a01, a0, a1);
@@ -397,7 +399,8 @@ __device__ __forceinline__ float group_sum_pipe(uint32_t tcol, uint32_t nc, floa
   return (a0 + a1) + (a2 + a3);
 }
 
-template <int D, bool LISTS>
+// NC: chunks of 16 columns of a group (P.RG / 16).
+template <int D, bool LISTS, int NC>
 __global__ void __launch_bounds__(NTHREADS, 1)
     mass_umma_kernel(const __grid_constant__ CUtensorMap kmap,
                       const __grid_constant__ CUtensorMap pmap, const __grid_constant__ Problem P,
@@ -590,14 +593,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           if (lane == 0) mbar_arrive(&tempty[buf]);
         };
         float* out = gdst + kt;
+#pragma unroll 1
         for (int gi = gb; gi < ge; ++gi, out += P.total_T) {
           const bool last = gi + 1 == ge && !my_anchor;
           auto loaded = [&] { if (last) release(); };
-          const uint32_t tcol = tacc + (uint32_t)(gi * P.RG), nc = cv + 4 * gi * P.RG;
-          float sm;
-          if (P.RG == 112) sm = group_sum_pipe<7>(tcol, nc, alpha, loaded);
-          else if (P.RG == 128) sm = group_sum_pipe<8>(tcol, nc, alpha, loaded);
-          else sm = group_sum(tcol, nc, P.RG, alpha, loaded);
+          const float sm = group_sum<NC>(tacc + (uint32_t)(gi * P.RG), cv + 4 * gi * P.RG, alpha, loaded);
           if (valid) *out = sm;
         }
         if (my_anchor) {
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           } else {
             // the r anchor rows, in 8-column steps (the padding rows up to 16
             // would add exp2(-inf) = 0)
-            const float sm = group_sum(tacc + (uint32_t)a0, cv + 4 * a0, (P.r + 7) & ~7, alpha, release);
+            const float sm = anchor_sum(tacc + (uint32_t)a0, cv + 4 * a0, (P.r + 7) & ~7, alpha, release);
             if (valid)
               bf.anchor[((size_t)x.l * P.Hkv + x.h) * P.total_T + col] = sm / (float)P.r;
           }
@@ -1171,38 +1171,41 @@ cudaError_t launch_softmax_only(const Problem& P, const Buffers& bf, cudaStream_
   return launch_softmax_d<D, true>(P, bf, st, kmap, pmap, nsm);
 }
 
+// Mass pass: workers are CTAs, one per SM. Groups of any width up to a block.
+template <int D, int NC = SROWS / 16>
+cudaError_t launch_mass(const Problem& P, const Buffers& bf, cudaStream_t st, const CUtensorMap& kmap,
+                        const CUtensorMap& pmap, int nsm) {
+  if constexpr (NC > 1)
+    if (P.RG < 16 * NC) return launch_mass<D, NC - 1>(P, bf, st, kmap, pmap, nsm);
+  cudaError_t e;
+  for (auto f : {mass_umma_kernel<D, false, NC>, mass_umma_kernel<D, true, NC>})
+    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  Smem<D>::DYN_BYTES)) != cudaSuccess) return e;
+  Sched s2 = make_sched(P, 2);
+  if (!s2.units) return cudaSuccess;
+  if (balance_workers(s2.wl, s2.ntiles, s2.units / s2.ntiles, nsm))
+    return launch_kernel(mass_umma_kernel<D, true, NC>, dim3(nsm), NTHREADS, Smem<D>::DYN_BYTES, st,
+                         P.overlap, 0, kmap, pmap, P, s2, bf);
+  const int rows = s2.units / s2.ntiles;
+  const int grid = std::max(1, std::min(nsm / s2.ntiles, rows)) * s2.ntiles;
+  return launch_kernel(mass_umma_kernel<D, false, NC>, dim3(grid), NTHREADS, Smem<D>::DYN_BYTES, st,
+                       P.overlap, 0, kmap, pmap, P, s2, bf);
+}
+
 template <int D>
 cudaError_t launch_d(const Problem& P, const Buffers& bf, cudaStream_t st, const void* K,
                      cudaEvent_t* ev) {
-  using SM = Smem<D>;
   CUtensorMap kmap, pmap;
   cudaError_t e = make_maps<D>(P, bf, K, &kmap, &pmap);
   if (e != cudaSuccess) return e;
   const int nsm = sm_count();
   if (nsm <= 0) return cudaErrorInvalidDevice;
-  for (auto f : {mass_umma_kernel<D, false>, mass_umma_kernel<D, true>})
-    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  SM::DYN_BYTES)) != cudaSuccess) return e;
-  Sched s2 = make_sched(P, 2);
   if (ev && (e = cudaEventRecord(ev[1], st)) != cudaSuccess) return e;
   if ((e = launch_softmax_d<D, false>(P, bf, st, kmap, pmap, nsm)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[2], st)) != cudaSuccess) return e;
   if ((e = launch_merge(P, bf, st)) != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[3], st)) != cudaSuccess) return e;
-  if (s2.units) {
-    // mass pass: workers are CTAs, one per SM
-    if (balance_workers(s2.wl, s2.ntiles, s2.units / s2.ntiles, nsm)) {
-      e = launch_kernel(mass_umma_kernel<D, true>, dim3(nsm), NTHREADS, SM::DYN_BYTES, st, P.overlap, 0,
-                        kmap, pmap, P, s2, bf);
-    } else {
-      const int rows = s2.units / s2.ntiles;
-      const int grid = std::max(1, std::min(nsm / s2.ntiles, rows)) * s2.ntiles;
-      e = launch_kernel(mass_umma_kernel<D, false>, dim3(grid), NTHREADS, SM::DYN_BYTES, st, P.overlap, 0,
-                        kmap, pmap, P, s2, bf);
-    }
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  return launch_mass<D>(P, bf, st, kmap, pmap, nsm);
 }
 
 }  // namespace
