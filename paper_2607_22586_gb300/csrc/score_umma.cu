@@ -1097,8 +1097,9 @@ Sched make_sched(const Problem& P, int pass) {
     s.ntiles = (P.anchor_split ? P.n_group_rows : P.Prows_pad) / SROWS;
   } else {
     // fewest blocks of whole groups, the last one with the anchor rows
-    const int per_block = SROWS / P.RG;                      // >= 1 (RG <= SROWS)
-    const int per_last = (SROWS - P.anchor_rows) / P.RG;     // >= 0
+    const int rg = std::max(P.RG, 1);                        // 0 without groups
+    const int per_block = SROWS / rg;                        // >= 1 (RG <= SROWS)
+    const int per_last = (SROWS - P.anchor_rows) / rg;       // >= 0
     s.last_groups = min(per_last, P.G);
     s.ntiles = 1 + (P.G - s.last_groups + per_block - 1) / per_block;
   }

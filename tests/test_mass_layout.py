@@ -27,7 +27,19 @@ HARNESS = r"""
 namespace mmshift { cudaError_t launch_merge(const Problem&, const Buffers&, cudaStream_t) { return cudaSuccess; } }
 using namespace mmshift;
 
-int main() {
+int main(int argc, char**) {
+  if (argc > 1) {   // no groups at all: one block of the anchor rows
+    for (int r : {1, 7, 16, 256}) {
+      Problem P;
+      memset(&P, 0, sizeof(P));
+      P.r = r; P.anchor_rows = ((r + 15) / 16) * 16;
+      P.B = 1; P.L = 1; P.Hkv = 1; P.req[0].nsplit = 1;
+      const Sched s = make_sched(P, 2);
+      const Block k = mass_block(P, s, 0);
+      std::printf("%d %d %d %d %d\n", s.ntiles, k.row0, k.rows, k.ng, k.anchor);
+    }
+    return 0;
+  }
   int checked = 0;
   for (int r : {1, 2, 4, 7, 8, 16})
     for (int gs : {1, 2, 4, 8, 16, 32, 64, 128, 256})
@@ -81,7 +93,7 @@ int main() {
 
 
 @pytest.fixture(scope="module")
-def output(tmp_path_factory):
+def harness(tmp_path_factory):
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     if not os.path.exists(nvcc):
         pytest.skip("nvcc not found")
@@ -91,7 +103,12 @@ def output(tmp_path_factory):
     subprocess.run([nvcc, "-std=c++17", "-O1", "-gencode", "arch=compute_103a,code=sm_103a",
                     "--expt-relaxed-constexpr", "-I", CSRC, "-I", os.path.join(ROOT, "include"),
                     str(src), "-o", str(exe)], check=True, capture_output=True)
-    out = subprocess.run([str(exe)], capture_output=True, text=True)
+    return str(exe)
+
+
+@pytest.fixture(scope="module")
+def output(harness):
+    out = subprocess.run([harness], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout[-2000:]
     return out.stdout
 
@@ -107,3 +124,11 @@ def test_benchmark_shapes(output):
     assert lines["r7G2"] == "240"
     assert lines["r8G32"] == " ".join(["256"] * 15 + ["128", "144"])
     assert lines["r8G2"] == "128 144"                            # no anchor-only block
+
+
+def test_the_anchor_alone(harness):
+    # a group has no rows to divide by
+    out = subprocess.run([harness, "none"], capture_output=True, text=True)
+    assert out.returncode == 0
+    assert [line.split() for line in out.stdout.split("\n")[:-1]] == [
+        ["1", "0", rows, "0", "1"] for rows in ("16", "16", "16", "256")]
