@@ -152,20 +152,6 @@ __device__ __forceinline__ float logit(const uint64_t (&acc)[8][4], int i, int j
   return (j & 1) ? hi : lo;
 }
 
-// Shared::cluster address of this CTA's shared-memory location in CTA `rank`,
-// and a 64-bit load from there.
-__device__ __forceinline__ float2 ld_cluster_f2(const float2* p, int rank) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-  uint32_t c;
-  float2 v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(c) : "r"(a), "r"(rank));
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(c) : "memory");
-  return v;
-}
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // RATIO: the sums feed a ratio (coverage), over at most bf.kept_len keys where
 // given; a NaN logit then makes its row's sum NaN, also where all logits of its
 // 16 keys are NaN, which the selection's maxima pass over.
@@ -270,21 +256,21 @@ __global__ void __launch_bounds__(TNT, 3) pass1_simt(const __grid_constant__ Pro
       }
     }
   }
-  if (nrank > 1) cluster_barrier(); else __syncthreads();
+  if (nrank > 1) umma::cluster_sync(); else __syncthreads();
   if (rank == 0 && tid < TR && rt * TR + tid < P.Prows_pad) {
     float run_m = -INFINITY, run_z = 0.f;
     for (int r = 0; r < nrank; ++r) {
       const int n = 2 * ((r + 1) * ntiles / nrank - r * ntiles / nrank);
       for (int i = 0; i < n; ++i) {
         const float2* p = pairs + (size_t)i * TR + tid;
-        const float2 v = r == 0 ? *p : ld_cluster_f2(p, r);
+        const float2 v = r == 0 ? *p : umma::ld_cluster_f2(umma::mapa(umma::smem_u32(p), (uint32_t)r));
         merge_ms(run_m, run_z, v.x, v.y);
       }
     }
     bf.part[(((size_t)l * P.Hkv + h) * P.total_splits + s) * P.part_slots * P.Prows_pad +
             rt * TR + tid] = make_float2(run_m, run_z);
   }
-  if (nrank > 1) cluster_barrier();   // no CTA leaves while the first may still read its pairs
+  if (nrank > 1) umma::cluster_sync();   // no CTA leaves while the first may still read its pairs
 }
 
 // SUB threads per row (four when a row has at least 128 partials, else one):

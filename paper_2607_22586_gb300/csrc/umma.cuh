@@ -260,10 +260,6 @@ __device__ __forceinline__ float2 ld_cluster_f2(uint32_t caddr) {
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(caddr) : "memory");
   return v;
 }
-// Arrive on an mbarrier of either CTA of the cluster (cluster address).
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t caddr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(caddr) : "memory");
-}
 // Relaxed arrival on an mbarrier of either CTA of the cluster: orders no
 // memory accesses, for releases whose data dependence is already complete
 // (e.g. tensor-memory reads finished by tcgen05.wait::ld).
