@@ -211,7 +211,12 @@ int choose_umma(const Problem& P, const void* K) {
 // 256-row blocks x heads x layers; 76 CTA pairs take them): its kernels are then
 // launched as programmatic dependents. One layer of 4096 keys (240 units) 108 ->
 // 96.5 us, steps 2-4 on 4,500 keys 53 -> 44 us, two layers of 8192 keys (960 units)
-// 185 -> 179.5 us; the 28-layer stacks (13,440 and 53,760 units) lose 1-2%.
+// 193.5 -> 185.7 us; the 28-layer stacks (13,440 and 53,760 units) lose 1-2 %. In
+// between both ways lie within 4 %: at 1,024 units eight layers of 32K keys with few
+// proxies lose 1.3 % and eight of 16K gain 0.8 %, at 1,536 to 2,048 the former lose
+// 1 to 1.6 % and three to six layers of 8192 keys gain 2 to 4 %, at 3,584 to 7,680
+// both gain 1 to 2 %, the 72B-class batch gains 0.5 to 4 % at 1,200 to 4,800 and
+// loses 1.8 % at 12,000: no other line is better for all.
 constexpr long long kShortCall = 1024;
 
 // Scoring path of a call: tensor or CUDA cores, and the softmax partials
@@ -771,8 +776,9 @@ mmshift_status mmshift_coverage(const mmshift_shape* s, const void* K, const voi
   if ((st = carve(P, workspace, workspace_bytes, &bf)) != MMSHIFT_OK) return st;
   const cudaStream_t cs = (cudaStream_t)stream;
   // two softmax passes where the copied kept rows fit in the workspace that
-  // steps 2-4 need (its size is the entry's contract either way): with 32
-  // decode queries, budgets up to about half the prompt
+  // steps 2-4 need (its size is the entry's contract either way): on 28 layers of
+  // 32K keys with 28 / 4 heads, budgets up to 71 % of the prompt with 32 decode
+  // queries, 16 % with 8, 6.25 % with two and 4.7 % with one
   CoverageJob J;
   coverage_job(P, &J);
   if (J.total <= layout_of(P).total)

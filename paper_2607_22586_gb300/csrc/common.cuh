@@ -14,10 +14,12 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kChunk = 16;       // proxy rows per packing chunk (one group id)
 constexpr int kRowTile = 256;    // proxy rows are padded to a multiple of this
 constexpr int kMaxSplitAnchor = 8;  // anchor_split needs r <= this (one warp per anchor row)
-// Key split length of the softmax pass. It is a constant, so the order in
-// which a request's partial (max, sum) pairs are merged -- and with it every
-// bit of the result -- does not depend on the other requests or layers of the
-// call.
+// Key split length of the softmax pass. It is a constant, so a request's partial
+// (max, sum) pairs do not depend on the other requests or layers of the call. The
+// order of their merge does not depend on the layers either, but on the longest
+// request: from 128 partials of a row on (32 splits on the tensor cores) four
+// chains take every row's partials, so a short request beside such a long one can
+// differ in the last bits from the same request alone.
 constexpr int kSplitLen = 1024;
 constexpr int kUmmaPartSlots = 4; // softmax partials per (row, split) of the tensor-core pass
 
