@@ -34,6 +34,10 @@
  *     host link. mmshift_select and mmshift_gather check K, Qwin and V
  *     with cudaPointerGetAttributes and refuse (MMSHIFT_ERR_INVALID_ARG)
  *     pageable host memory.
+ *   - A buffer starts at an address that is a multiple of its elements' size,
+ *     more where its entry says so. Bases and layer strides of multiples of 16
+ *     bytes are the fast ones (K of a bfloat16 call needs them for the tensor
+ *     cores).
  *   - All work is enqueued on `stream` (a cudaStream_t; NULL is the legacy
  *     default stream) and is asynchronous.
  *   - Host-side validation runs first; on error nothing is enqueued and the

@@ -195,6 +195,28 @@ __device__ __forceinline__ void set_status(int* status, int bit) {
   if (status) atomicOr(status, bit);
 }
 
+// 16 bytes of an input row, and of an output row; `vec`: the addresses allow one
+// access, else they are those of 16-bit or larger elements.
+__device__ __forceinline__ uint4 load_row16(const uint8_t* p, bool vec) {
+  if (vec) return __ldg(reinterpret_cast<const uint4*>(p));
+  const uint16_t* q = reinterpret_cast<const uint16_t*>(p);
+  return make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16,
+                    q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16);
+}
+__device__ __forceinline__ void store_row16(uint8_t* p, const uint4& v, bool vec) {
+  if (vec) {
+    *reinterpret_cast<uint4*>(p) = v;
+    return;
+  }
+  uint16_t* q = reinterpret_cast<uint16_t*>(p);
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    q[2 * i] = (uint16_t)w[i];
+    q[2 * i + 1] = (uint16_t)(w[i] >> 16);
+  }
+}
+
 // Start of every kernel that may be launched as a programmatic dependent: the
 // next kernel of the call may take its place on the SMs, and everything the
 // kernels before this one wrote is visible afterwards. Without the launch

@@ -135,15 +135,7 @@ __global__ void __launch_bounds__(KRT) kept_rows_kernel(const __grid_constant__ 
 #pragma unroll 4
   for (int e = tid / LPR; e < n; e += KRT / LPR) {
     const uint8_t* p = src + (size_t)list[e] * rstride + part * 16;
-    uint4 v;
-    if (vec) {
-      v = __ldg(reinterpret_cast<const uint4*>(p));
-    } else {                       // keys at an address no 16-byte load takes
-      const uint16_t* q = reinterpret_cast<const uint16_t*>(p);
-      v = make_uint4(q[0] | (uint32_t)q[1] << 16, q[2] | (uint32_t)q[3] << 16,
-                     q[4] | (uint32_t)q[5] << 16, q[6] | (uint32_t)q[7] << 16);
-    }
-    *reinterpret_cast<uint4*>(dst + (size_t)e * rstride + part * 16) = v;
+    *reinterpret_cast<uint4*>(dst + (size_t)e * rstride + part * 16) = load_row16(p, vec);
   }
 }
 

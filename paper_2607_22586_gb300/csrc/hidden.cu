@@ -119,19 +119,23 @@ __device__ __forceinline__ void rotate(float& x, float& y, float cs, float sn) {
   x = a * cs - e * sn;
   y = e * cs + a * sn;
 }
-__device__ __forceinline__ void store16_bf16(__nv_bfloat16* dst, const float (&x)[16], bool vec) {
+// align: of dst, as far as it matters (16, 8 or less).
+__device__ __forceinline__ void store16_bf16(__nv_bfloat16* dst, const float (&x)[16], int align) {
   uint32_t u[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(x[2 * k], x[2 * k + 1]);
     u[k] = *reinterpret_cast<const uint32_t*>(&p);
   }
-  if (vec) {
+  if (align == 16) {
     reinterpret_cast<uint4*>(dst)[0] = make_uint4(u[0], u[1], u[2], u[3]);
     reinterpret_cast<uint4*>(dst)[1] = make_uint4(u[4], u[5], u[6], u[7]);
-  } else {
+  } else if (align == 8) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) reinterpret_cast<uint2*>(dst)[k] = make_uint2(u[2 * k], u[2 * k + 1]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) dst[k] = __float2bfloat16_rn(x[k]);
   }
 }
 
@@ -146,7 +150,9 @@ __device__ __forceinline__ void drain_tile(const HiddenJob& J, int lb, int nt, i
   const float* rope = J.rope ? J.rope + (size_t)b * D : nullptr;   // [d/2][2]
   // 16-byte bias loads and stores where the caller's addresses allow them
   const bool bvec = (reinterpret_cast<uintptr_t>(bias) & 15) == 0;
-  const bool ovec = (reinterpret_cast<uintptr_t>(J.out) & 15) == 0;
+  const int oalign = (reinterpret_cast<uintptr_t>(J.out) & 15) == 0  ? 16
+                     : (reinterpret_cast<uintptr_t>(J.out) & 7) == 0 ? 8
+                                                                     : 2;
   for (int hh = 0; hh < J.NT / D; ++hh) {
     const int hq = nt * (J.NT / D) + hh;
     __nv_bfloat16* dst = J.out + ((((size_t)l * J.B + b) * J.Hq + hq) * J.N + m) * D;
@@ -169,8 +175,8 @@ __device__ __forceinline__ void drain_tile(const HiddenJob& J, int lb, int nt, i
         }
       }
       if (valid) {
-        store16_bf16(dst + c, x, ovec);
-        store16_bf16(dst + D / 2 + c, y, ovec);
+        store16_bf16(dst + c, x, oalign);
+        store16_bf16(dst + D / 2 + c, y, oalign);
       }
     }
   }

@@ -47,7 +47,15 @@ __device__ __forceinline__ void normals8(const Problem& P, int i, int q, int hq,
               z);
 }
 
-// Four consecutive values rounded to T, one vector store.
+// Four consecutive values rounded to T, one vector store or, where the caller's
+// address does not allow it, four.
+template <typename T>
+__device__ __forceinline__ void store1x4(T* dst, float a, float b, float c, float d) {
+  dst[0] = from_f32<T>(a);
+  dst[1] = from_f32<T>(b);
+  dst[2] = from_f32<T>(c);
+  dst[3] = from_f32<T>(d);
+}
 __device__ __forceinline__ void store4(__nv_bfloat16* dst, float a, float b, float c, float d) {
   __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
   uint2 u;
@@ -396,8 +404,14 @@ __global__ void __launch_bounds__(256, 6) proxy_pack_kernel(Problem P, Buffers b
       store4(dst + D / 2 + 4 * qq, v[4], v[5], v[6], v[7]);
     }
     if (pout) {
-      store4(pout + (size_t)i * D + 4 * qq, v[0], v[1], v[2], v[3]);
-      store4(pout + (size_t)i * D + D / 2 + 4 * qq, v[4], v[5], v[6], v[7]);
+      T* dst = pout + (size_t)i * D + 4 * qq;
+      if ((reinterpret_cast<uintptr_t>(dst) & (4 * sizeof(T) - 1)) == 0) {
+        store4(dst, v[0], v[1], v[2], v[3]);
+        store4(dst + D / 2, v[4], v[5], v[6], v[7]);
+      } else {
+        store1x4(dst, v[0], v[1], v[2], v[3]);
+        store1x4(dst + D / 2, v[4], v[5], v[6], v[7]);
+      }
     }
   }
   if (!packed) return;

@@ -1446,7 +1446,8 @@ template <int ROWB>
 __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Problem P,
                                                      const __grid_constant__ Buffers bf,
                                                      const uint8_t* K, const uint8_t* V,
-                                                     const int32_t* idx, uint8_t* oK, uint8_t* oV) {
+                                                     const int32_t* idx, uint8_t* oK, uint8_t* oV,
+                                                     bool vec_in, bool vec_out) {
   dependent_start();
   constexpr int LPR = ROWB / 16;  // lanes per row
   const int l = blockIdx.y;
@@ -1459,18 +1460,18 @@ __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ Pro
   const ReqInfo R = P.req[b];
   const int t = idx[(size_t)l * P.R * P.Hkv + q];
   const size_t esz = ROWB / P.d;
-  uint4* dk = (uint4*)(oK + (((size_t)l * P.R * P.Hkv + q) * ROWB)) + part;
-  uint4* dv = (uint4*)(oV + (((size_t)l * P.R * P.Hkv + q) * ROWB)) + part;
+  const size_t dst = ((size_t)l * P.R * P.Hkv + q) * ROWB + part * 16;
   if (t < 0 || t >= R.t_len) {
     // zero rows: padding of a head with its own smaller budget (-1), or a bad index
-    *dk = make_uint4(0, 0, 0, 0);
-    *dv = make_uint4(0, 0, 0, 0);
+    store_row16(oK + dst, make_uint4(0, 0, 0, 0), vec_out);
+    store_row16(oV + dst, make_uint4(0, 0, 0, 0), vec_out);
     if (part == 0 && !(bf.head_budget && t == -1)) set_status(bf.status, kStatusBadIndex);
     return;
   }
   const size_t src = (size_t)l * P.ls_kv * esz + (((size_t)R.tok_off + t) * P.Hkv + h) * ROWB;
-  *dk = __ldg((const uint4*)(K + src) + part);
-  *dv = __ldg((const uint4*)(V + src) + part);
+  const uint4 k = load_row16(K + src + part * 16, vec_in), v = load_row16(V + src + part * 16, vec_in);
+  store_row16(oK + dst, k, vec_out);
+  store_row16(oV + dst, v, vec_out);
 }
 
 }  // namespace
@@ -1560,13 +1561,17 @@ cudaError_t launch_gather(const Problem& P, const Buffers& bf, cudaStream_t st, 
   const int rowb = P.d * (P.dtype == MMSHIFT_BF16 ? 2 : 4);
   const long long rows = (long long)P.R * P.Hkv;
   if (rows == 0) return cudaSuccess;
+  const size_t esz = P.dtype == MMSHIFT_BF16 ? 2 : 4;
+  auto at = [](const void* p) { return reinterpret_cast<uintptr_t>(p); };
+  const bool vec_in = ((at(K) | at(V) | (uintptr_t)(P.ls_kv * esz)) & 15) == 0;
+  const bool vec_out = ((at(outK) | at(outV)) & 15) == 0;
 #define MMSHIFT_GATHER(RB)                                                                   \
   {                                                                                          \
     constexpr int LPR = RB / 16;                                                             \
     dim3 grid((unsigned)((rows + (256 / LPR) - 1) / (256 / LPR)), P.L);                      \
     return launch_kernel(gather_kernel<RB>, grid, 256, 0, st, P.overlap, 0, P, bf,            \
                          (const uint8_t*)K, (const uint8_t*)V, idx, (uint8_t*)outK,          \
-                         (uint8_t*)outV);                                                    \
+                         (uint8_t*)outV, vec_in, vec_out);                                   \
   }
   switch (rowb) {
     case 128: MMSHIFT_GATHER(128)
