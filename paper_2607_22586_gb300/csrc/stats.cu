@@ -6,7 +6,7 @@
 // A streaming reduction over Q [L][total_T][Hq][d]: every byte of Q is read
 // once, in coalesced 16-byte vectors, so the pass is bounded by HBM.
 //  - stats_partial_kernel: a chunk of kStatsChunk prompt queries of one request
-//    and layer, one thread per 8 consecutive columns (q-head, dimension), 64
+//    and layer, one thread per 16 bytes of columns (q-head, dimension), 64
 //    threads per CTA so that a few hundred chunks fill the SMs evenly; a thread
 //    keeps, per column, the sums of (x - x0) and (x - x0)^2 in fp32, x0 being
 //    the chunk's first query (the shift keeps the second sum free of
@@ -15,6 +15,10 @@
 //    and one CTA of 448 threads per chunk the compiler and the uneven waves left
 //    fewer in flight: 940 MB of hidden states 179 -> 163 us (both kernels), 6.6
 //    GB of prompt queries 1,065 -> 952 us, 6.9 TB/s. 128 threads: 180 us.
+//    Float32 threads take four columns: with eight, as two copies of 16 bytes, a
+//    warp's accesses leave every other 16 bytes out and each sector is fetched
+//    twice (1.07 GB of hidden states 228 us before the copies, 347 with eight
+//    columns, 178 with four).
 //  - stats_merge_kernel: one thread per column merges the chunks in order with
 //    the pairwise update of Chan, Golub and LeVeque (count, mean, sum of
 //    squared deviations), then writes mean and std.
@@ -26,29 +30,24 @@ namespace mmshift {
 namespace {
 
 constexpr int kStatsGroup = 4;     // rows per asynchronous copy group
-constexpr int kStatsRing = 8;      // groups in flight per thread (bf16; half as many in float32)
-constexpr int kStatsThreads = 64;  // column groups (of eight columns) per CTA
+constexpr int kStatsRing = 8;      // groups in flight per thread
+constexpr int kStatsThreads = 64;  // column groups (of 16 bytes a row) per CTA
 constexpr int kMergeAhead = 8;     // chunks of partial sums loaded ahead in the merge
 
-// 16-byte words of eight elements as float32.
-template <typename T>
-constexpr int kWords = 8 * (int)sizeof(T) / 16;
-__device__ __forceinline__ void unpack8(const uint4 (&v)[1], float (&x)[8]) {
-  const uint32_t w[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+// The 16 / sizeof(T) elements of a 16-byte word as float32.
+__device__ __forceinline__ void unpack(const uint4& v, float (&x)[8]) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     x[2 * i] = __uint_as_float(w[i] << 16);
     x[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
   }
 }
-__device__ __forceinline__ void unpack8(const uint4 (&v)[2], float (&x)[8]) {
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    x[4 * i] = __uint_as_float(v[i].x);
-    x[4 * i + 1] = __uint_as_float(v[i].y);
-    x[4 * i + 2] = __uint_as_float(v[i].z);
-    x[4 * i + 3] = __uint_as_float(v[i].w);
-  }
+__device__ __forceinline__ void unpack(const uint4& v, float (&x)[4]) {
+  x[0] = __uint_as_float(v.x);
+  x[1] = __uint_as_float(v.y);
+  x[2] = __uint_as_float(v.z);
+  x[3] = __uint_as_float(v.w);
 }
 
 __device__ __forceinline__ void copy16(void* smem, const void* gmem) {
@@ -64,8 +63,8 @@ __device__ __forceinline__ void copy16(void* smem, const void* gmem) {
 template <typename T>
 __global__ void __launch_bounds__(kStatsThreads) stats_partial_kernel(const __grid_constant__ StatsJob J,
                                                                      const T* Q, float* part, int ncp) {
-  constexpr int W = kWords<T>, G = kStatsGroup, NG = kStatsRing / W;
-  extern __shared__ uint4 ring[];    // [NG][G][W][blockDim.x]
+  constexpr int C = 16 / (int)sizeof(T), G = kStatsGroup, NG = kStatsRing;   // C: columns per thread
+  extern __shared__ uint4 ring[];    // [NG][G][blockDim.x]
   const int c = blockIdx.x / ncp, cp = blockIdx.x % ncp, b = blockIdx.y, l = blockIdx.z;
   const int t_len = J.t_len[b];
   const int t0 = c * kStatsChunk;
@@ -74,42 +73,30 @@ __global__ void __launch_bounds__(kStatsThreads) stats_partial_kernel(const __gr
   const T* q = Q + (size_t)l * J.ls + ((size_t)J.tok_off[b] + t0) * J.ncol;
   float* out = part + (((size_t)l * J.B + b) * J.nchunk + c) * 3 * J.ncol;
   const int nt = blockDim.x;
-  for (int cg = cp * nt + threadIdx.x; cg < J.ncol / 8; cg += ncp * nt) {
-    const T* col = q + (size_t)cg * 8;
+  for (int cg = cp * nt + threadIdx.x; cg < J.ncol / C; cg += ncp * nt) {
+    const T* col = q + (size_t)cg * C;
     // rows 1 .. n - 1 in groups of G, NG groups on their way to this thread's
     // own places of the ring (no other thread reads them, so no barrier)
-    auto slot = [&](int g, int u, int w) { return ring + ((size_t)(g * G + u) * W + w) * nt + threadIdx.x; };
+    auto slot = [&](int g, int u) { return ring + (size_t)(g * G + u) * nt + threadIdx.x; };
     auto fetch = [&](int g) {
 #pragma unroll
       for (int u = 0; u < G; ++u) {
         const int t = 1 + g * G + u;
-        if (t < n) {
-#pragma unroll
-          for (int w = 0; w < W; ++w)
-            copy16(slot(g % NG, u, w), reinterpret_cast<const uint4*>(col + (size_t)t * J.ncol) + w);
-        }
+        if (t < n) copy16(slot(g % NG, u), col + (size_t)t * J.ncol);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
 #pragma unroll 1
     for (int g = 0; g < NG; ++g) fetch(g);
-    float x0[8], s1[8], s2[8];
-    {
-      uint4 v[W];
+    float x0[C], s1[C], s2[C];
+    unpack(__ldg(reinterpret_cast<const uint4*>(col)), x0);
 #pragma unroll
-      for (int w = 0; w < W; ++w) v[w] = __ldg(reinterpret_cast<const uint4*>(col) + w);
-      unpack8(v, x0);
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) { s1[k] = 0.f; s2[k] = 0.f; }
+    for (int k = 0; k < C; ++k) { s1[k] = 0.f; s2[k] = 0.f; }
     auto add = [&](int g, int u) {
-      uint4 v[W];
+      float x[C];
+      unpack(*slot(g, u), x);
 #pragma unroll
-      for (int w = 0; w < W; ++w) v[w] = *slot(g, u, w);
-      float x[8];
-      unpack8(v, x);
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
+      for (int k = 0; k < C; ++k) {
         const float dv = x[k] - x0[k];
         s1[k] += dv;
         s2[k] = fmaf(dv, dv, s2[k]);
@@ -127,10 +114,10 @@ __global__ void __launch_bounds__(kStatsThreads) stats_partial_kernel(const __gr
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      out[cg * 8 + k] = x0[k];
-      out[J.ncol + cg * 8 + k] = s1[k];
-      out[2 * J.ncol + cg * 8 + k] = s2[k];
+    for (int k = 0; k < C; ++k) {
+      out[cg * C + k] = x0[k];
+      out[J.ncol + cg * C + k] = s1[k];
+      out[2 * J.ncol + cg * C + k] = s2[k];
     }
   }
 }
@@ -177,8 +164,9 @@ __global__ void __launch_bounds__(256) stats_merge_kernel(StatsJob J, const floa
 
 cudaError_t launch_prefill_stats(const StatsJob& J, const void* Q, float* part, float* stats,
                                  cudaStream_t st, bool bf16) {
-  const int threads = std::min(kStatsThreads, (J.ncol / 8 + 31) / 32 * 32);
-  const int ncp = (J.ncol / 8 + threads - 1) / threads;
+  const int groups = J.ncol / (bf16 ? 8 : 4);
+  const int threads = std::min(kStatsThreads, (groups + 31) / 32 * 32);
+  const int ncp = (groups + threads - 1) / threads;
   dim3 g1(J.nchunk * ncp, J.B, J.L);
   const size_t smem = (size_t)kStatsRing * kStatsGroup * threads * 16;
   cudaError_t e;

@@ -1,5 +1,6 @@
 """mmshift_hidden_stats at the edges of its chunks (512 rows), of the copy
-groups (4 rows, 32 ahead) and of a CTA's columns (64 threads of eight):
+groups (4 rows, 32 ahead) and of a CTA's columns (64 threads of eight, in float32
+of four):
 compared with float64 in plain torch under the bounds of the statistics tests
 (fp32 sums shifted by the chunk's first row, chunks merged pairwise: mean within
 5e-5 (|mean| + std), std within 2e-4 std + 1e-6 |mean|)."""
@@ -12,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("lens", [(1, 2, 3), (4, 5, 6, 33, 34), (36, 37, 511), (512, 513, 514), (1025, 1600)])
-@pytest.mark.parametrize("ncol,dtype", [(64, "bf16"), (520, "bf16"), (3584, "bf16"), (264, "f32")])
+@pytest.mark.parametrize("ncol,dtype", [(64, "bf16"), (520, "bf16"), (3584, "bf16"), (8, "f32"), (264, "f32"),
+                                        (2056, "f32")])
 def test_statistics_at_edges(lens, ncol, dtype):
     dt = torch.bfloat16 if dtype == "bf16" else torch.float32
     gen = torch.Generator(device="cuda").manual_seed(sum(lens) + ncol)
