@@ -582,9 +582,13 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
   const int draws = P.Np * (D / 8);
   int nch = draws <= 0 ? 1 : std::min(kProxyChunks, (draws + 1023) / 1024);
   // a short call's heads are spread further, down to one draw per thread,
-  // until the launch holds the six CTAs per SM that fit
+  // until the launch holds the six CTAs per SM that fit; rotated, two per SM: each
+  // CTA works out the rotation's angles in float64, which more of them wait for
+  // (one layer of 28 heads, N = 512, rotated, from given statistics: 16.6 us with up
+  // to three, 20.9 with six; sampler and refinement from a window 35 and 44)
   const long long heads = (long long)P.Hq * P.B * P.L;
-  nch = (int)std::max<long long>(nch, std::min<long long>((draws + 255) / 256, 6LL * nsm / heads));
+  const bool rope = P.rope_theta > 0.f && !bf.proxies_in;
+  nch = (int)std::max<long long>(nch, std::min<long long>((draws + 255) / 256, (rope ? 2LL : 6LL) * nsm / heads));
   const bool refine = samples_bf16(P, bf);
   Buffers b2 = bf;
   if (!has_refine_list(bf)) {
@@ -597,7 +601,7 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
       (e = cudaMemsetAsync(b2.refine_count, 0, sizeof(int), st)) != cudaSuccess)
     return e;
   dim3 grid(P.Hq * nch, P.B, P.L);
-  if (P.rope_theta > 0.f && !bf.proxies_in)
+  if (rope)
     proxy_pack_kernel<T, D, true><<<grid, 256, 0, st>>>(P, b2, (const T*)qwin, nch);
   else
     proxy_pack_kernel<T, D, false><<<grid, 256, 0, st>>>(P, b2, (const T*)qwin, nch);
