@@ -174,16 +174,17 @@ __global__ void __launch_bounds__(128) ratio_runs_kernel(const __grid_constant__
   *src = make_float2(m, z);
 }
 
-// CTA = 32 decode queries of one (layer, request, KV head): thread (i, jj) merges
-// the partials of query i under query heads jj, jj + 8, ...; run, run_k: partials
-// already merged into each place that holds one.
-__global__ void __launch_bounds__(256) ratio_kernel(const __grid_constant__ Problem P,
+// CTA = NQ decode queries of one (layer, request, KV head): thread (i, jj) merges
+// the partials of query i under query heads jj, jj + nj, ..., nj = blockDim.x / NQ;
+// run, run_k: partials already merged into each place that holds one.
+template <int NQ>
+__global__ void __launch_bounds__(1024) ratio_kernel(const __grid_constant__ Problem P,
                                                     const __grid_constant__ Problem Pk,
                                                     const float2* all, const float2* kept,
                                                     int run, int run_k, float* cov) {
-  __shared__ float red[8][33];
-  const int li = threadIdx.x % 32, jj = threadIdx.x / 32;
-  const int i = blockIdx.x * 32 + li, h = blockIdx.y;
+  __shared__ float red[1024 / NQ][NQ + 1];
+  const int li = threadIdx.x % NQ, jj = threadIdx.x / NQ, nj = blockDim.x / NQ;
+  const int i = blockIdx.x * NQ + li, h = blockIdx.y;
   const int l = blockIdx.z / P.B, b = blockIdx.z % P.B;
   float share = 0.f;
   if (i < P.Np) {
@@ -193,7 +194,7 @@ __global__ void __launch_bounds__(256) ratio_kernel(const __grid_constant__ Prob
       const int ns = Q.req[b].nsplit * Q.part_slots;
       merge_run(src, (size_t)step * Q.Prows_pad, (ns + step - 1) / step, m, z);
     };
-    for (int j = jj; j < P.r; j += 8) {
+    for (int j = jj; j < P.r; j += nj) {
       float m = -INFINITY, z = 0.f, mk = -INFINITY, zk = 0.f;
       merged(P, all, run, j * P.gs + i, m, z);
       merged(Pk, kept, run_k, j * P.gs + i, mk, zk);
@@ -207,8 +208,7 @@ __global__ void __launch_bounds__(256) ratio_kernel(const __grid_constant__ Prob
   __syncthreads();
   if (jj == 0 && i < P.Np) {
     float s = 0.f;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s += red[k][li];
+    for (int k = 0; k < nj; ++k) s += red[k][li];
     cov[(((size_t)l * P.B + b) * P.Hkv + h) * P.Np + i] = s >= 0.f ? s / (float)P.r : 0.f;
   }
 }
@@ -253,8 +253,15 @@ cudaError_t launch_coverage_ratio(const Problem& P, const Problem& Pk, float2* a
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  ratio_kernel<<<dim3((P.Np + 31) / 32, P.Hkv, P.L * P.B), 256, 0, st>>>(P, Pk, all, kept, run[0], run[1],
-                                                                        cov);
+  // all query heads of a KV head side by side, up to 128 (32 queries, 128 heads over
+  // one KV head, 4096 keys: 125 us a call with eight at a time, 65 with 32, 51 so)
+  const int heads = (P.r + 7) / 8 * 8;
+  if (heads <= 32)
+    ratio_kernel<32><<<dim3((P.Np + 31) / 32, P.Hkv, P.L * P.B), 32 * heads, 0, st>>>(
+        P, Pk, all, kept, run[0], run[1], cov);
+  else
+    ratio_kernel<8><<<dim3((P.Np + 7) / 8, P.Hkv, P.L * P.B), 8 * min(128, heads), 0, st>>>(
+        P, Pk, all, kept, run[0], run[1], cov);
   return cudaGetLastError();
 }
 

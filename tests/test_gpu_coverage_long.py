@@ -3,7 +3,8 @@ on the tensor cores, one on the CUDA cores) are merged in runs of 64 first where
 they exceed one run: just below and above one run, last runs of one partial, short
 requests beside long ones, in the prompt's sums and in the kept rows' as well. The
 kept rows of budgets above 16,384 are placed by their chunks' counts: one more
-than that, several requests and layers, padding rows anywhere. Reference and bounds as in the tests of the kept rows."""
+than that, several requests and layers, padding rows anywhere. The query heads of a
+KV head are merged side by side, 8 to 128 of them. Reference and bounds as in the tests of the kept rows."""
 import math
 
 import pytest
@@ -54,4 +55,15 @@ def test_coverage_of_long_prompts(lens, budgets, hq, hkv, d, L, n_dec, dtype):
     ((40000, 300), (16640, 257), 4, 1, 64, 1, 70, "f32"),
 ])
 def test_coverage_of_large_budgets(lens, budgets, hq, hkv, d, L, n_dec, dtype):
+    _check(lens, budgets, hq, hkv, d, L, n_dec, dtype)
+
+
+@pytest.mark.parametrize("lens,budgets,hq,hkv,d,L,n_dec,dtype", [
+    ((900, 30), (100, 3), 18, 2, 64, 1, 33, "bf16"),            # nine heads: 16 places
+    ((700,), (50,), 32, 1, 128, 2, 5, "bf16"),
+    ((700,), (50,), 33, 1, 64, 1, 9, "bf16"),                   # eight queries a CTA
+    ((500, 1500), (20, 90), 128, 1, 64, 1, 33, "bf16"),
+    ((600,), (40,), 136, 1, 64, 1, 4, "bf16"),                  # two rounds
+])
+def test_coverage_of_many_query_heads(lens, budgets, hq, hkv, d, L, n_dec, dtype):
     _check(lens, budgets, hq, hkv, d, L, n_dec, dtype)
