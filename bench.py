@@ -61,18 +61,18 @@ SFU_EX2_PER_SM_CLK = 32          # MUFU.EX2 lanes per SM per clock on GB300 (mea
 # DRAM traffic (read + write) of the two scoring kernels per launch of the
 # default workload: one ncu capture of a 4-layer slice (one kernel launch each),
 # scaled by 7 to the 28 layers (the passes' units grow in proportion to the
-# layers; read per launch, of K's bytes: softmax pass 1.19x, mass pass 1.22x in
+# layers; read per launch, of K's bytes: softmax pass 1.17x, mass pass 1.22x in
 # the slice). It describes only the score_umma.cu it was measured on (checked by
 # hash).
-SCORE_TRAFFIC = {"source_sha256_16": "5514caf921f23a02", "workload": "qwen7b-28l-32k",
-                 "proxies": "paper", "softmax_pass": 7 * (159.062016e6 + 41.764864e6),
-                 "mass_pass": 7 * (163.506688e6 + 55.370240e6)}
+SCORE_TRAFFIC = {"source_sha256_16": "5acdcb67c02668ad", "workload": "qwen7b-28l-32k",
+                 "proxies": "paper", "softmax_pass": 7 * (156.355328e6 + 42.547712e6),
+                 "mass_pass": 7 * (163.975680e6 + 55.691008e6)}
 # DRAM traffic of the prompt-query statistics pass (both kernels) per launch
 # of the default workload, from one ncu capture of a 4-layer slice scaled by 7
-# (partial kernel 939.575552 MB read + 9.028608 MB written, merge 11.026432 MB
+# (partial kernel 939.564544 MB read + 9.113856 MB written, merge 11.026176 MB
 # read); valid for the stats.cu it was measured on (checked by hash).
-STATS_TRAFFIC = {"source_sha256_16": "38814d5537c1ac52", "workload": "qwen7b-28l-32k",
-                 "bytes": 7 * (939.575552e6 + 9.028608e6 + 11.026432e6)}
+STATS_TRAFFIC = {"source_sha256_16": "4e41aed56a87fda0", "workload": "qwen7b-28l-32k",
+                 "bytes": 7 * (939.564544e6 + 9.113856e6 + 11.026176e6)}
 UNIT = "tokens/s/layer"
 SM_COUNT = 152
 FP32_LANES_PER_SM = 128
