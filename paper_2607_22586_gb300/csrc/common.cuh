@@ -106,7 +106,7 @@ struct Buffers {
   // bf16 proxies whose float32 value lies too close to a rounding boundary
   // are recomputed in float64 (proxy.cu): the sampler appends them here and a
   // second kernel redoes them; without a list (null) it redoes every element
-  int* refine_count;          // entries appended (may exceed refine_cap)
+  unsigned long long* refine_count;   // entries appended (may exceed refine_cap)
   uint32_t* refine_items;     // [refine_cap] (layer * B + request, query head, proxy * d + dim), packed
   float* refine_stats;        // [L][B][Hq][5][d] exact window sums (x0, S1 hi / lo, S2 hi / lo)
   int32_t refine_cap;

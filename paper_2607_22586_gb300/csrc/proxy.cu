@@ -252,14 +252,15 @@ int bits_for(int64_t n) {   // values 0 .. n - 1
 // Appends the undecided elements (bit k: element k of the thread's draw) of
 // proxy i to the refinement list, with one atomic for the thread's. The count
 // keeps growing past the list's capacity, which tells refine_kernel to redo the
-// whole call.
+// whole call (64-bit: more elements than a 32-bit one holds would bring it round to
+// the list's beginning).
 template <int D>
 __device__ __noinline__ void enlist(const Problem& P, const Buffers& bf, int l, int b, int hq,
                                     int i, int qq, uint32_t undecided) {
-  int slot = atomicAdd(bf.refine_count, __popc(undecided));
+  unsigned long long slot = atomicAdd(bf.refine_count, (unsigned long long)__popc(undecided));
   const uint64_t e0 = ((uint64_t)(l * P.B + b) << bf.refine_lb_bit) |
                       ((uint64_t)hq << bf.refine_hq_bit) | (uint64_t)(i * D);
-  for (; undecided && slot < bf.refine_cap; ++slot) {
+  for (; undecided && slot < (unsigned)bf.refine_cap; ++slot) {
     const int k = __ffs(undecided) - 1;
     undecided &= undecided - 1;
     const uint64_t e = e0 | (k < 4 ? 4 * qq + k : D / 2 + 4 * qq + (k - 4));
@@ -509,8 +510,9 @@ __global__ void __launch_bounds__(224) refine_kernel(const __grid_constant__ Pro
   constexpr int half = D / 2;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const bool rope = P.rope_theta > 0.f;
-  const int cnt = *bf.refine_count;
-  if (cnt > bf.refine_cap) {
+  const unsigned long long count = *bf.refine_count;
+  const int cnt = (int)count;
+  if (count > (unsigned)bf.refine_cap) {
     refine_every<D>(P, bf, qwin);
     return;
   }
@@ -598,7 +600,7 @@ cudaError_t launch_t(const Problem& P, const Buffers& bf, cudaStream_t st, const
     b2.refine_stats = nullptr;
   }
   if (refine && b2.refine_items &&
-      (e = cudaMemsetAsync(b2.refine_count, 0, sizeof(int), st)) != cudaSuccess)
+      (e = cudaMemsetAsync(b2.refine_count, 0, sizeof(*b2.refine_count), st)) != cudaSuccess)
     return e;
   dim3 grid(P.Hq * nch, P.B, P.L);
   if (rope)
@@ -630,7 +632,7 @@ size_t proxy_refine_bytes(const Problem& P) {
 }
 
 void set_refine_list(const Problem& P, char* count, float* stats, Buffers* bf) {
-  bf->refine_count = reinterpret_cast<int*>(count);
+  bf->refine_count = reinterpret_cast<unsigned long long*>(count);
   bf->refine_items = reinterpret_cast<uint32_t*>(count + 256);
   bf->refine_stats = stats;
   bf->refine_hq_bit = bits_for((int64_t)P.Np * P.d);   // d is a power of two
